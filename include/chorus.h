@@ -176,7 +176,7 @@ chorus_status chorus_rk_step(chorus_mesh mesh, const chorus_params* params, chor
  * This is the end-to-end form of a step for callers whose state lives on the host.  In the FP32 form
  * the state is copied in by eight element ranges (on a stream of the mesh's own, after the work
  * already queued on `stream`), each range's face traces computed as soon as it has arrived, and the
- * last stage's residual runs on the same ranges, each range's new state copied back while the next is
+ * last stage's update runs on the same ranges, each range's new state copied back while the next is
  * computed; the result equals chorus_rk_step's bit for bit.  Calls on one mesh must not overlap. */
 chorus_status chorus_rk_step_host(chorus_mesh mesh, const chorus_params* params, chorus_precision prec,
                                   void* Q_host, void* Q_dev, void* workspace, double dt, int64_t n_steps,
@@ -279,8 +279,9 @@ chorus_status chorus_closure_attach(chorus_mesh coarse, const void* weights);
 /* Kernel timing for measurement.  While enabled, every kernel that chorus_residual and
  * chorus_rk_step launch is bracketed by a pair of CUDA events recorded on the call's stream (the
  * kernels themselves are unchanged).  chorus_timing_read synchronises the stream and returns, per
- * kernel class (0: face traces, 1: lifted gradients / one-sided viscous fluxes / wall fluxes,
- * 2: residual and RK update, 3: common fluxes of the interior faces), the summed device
+ * kernel class (0: face traces, 1: the volume kernel - lifted gradients, one-sided viscous face fluxes,
+ * interior fluxes, sources and RK combination, 2: the end-point fluxes added and the new state's
+ * traces, 3: common fluxes of the faces), the summed device
  * milliseconds and launch counts recorded since the last read, then clears them.  ms, counts: host
  * arrays of 4.  enable = 0 stops recording. */
 chorus_status chorus_timing_enable(chorus_mesh mesh, int enable);
@@ -291,7 +292,7 @@ chorus_status chorus_timing_read(chorus_mesh mesh, void* stream, double* ms, int
  * need a residual - for example an application that has handed all device memory to its own pool
  * allocator, or a latency-critical loop that must not call cudaMalloc (which can synchronise the
  * device).  They pass only the state Q and the output R (device, layout above); the scratch (face
- * traces, one-sided viscous face fluxes, gradient record, common face fluxes) lives in one fixed
+ * traces, one-sided viscous face fluxes, common face fluxes) lives in one fixed
  * 32 MiB device array
  * inside the library, which every GPU that loads the library holds until the process exits.
  *  - Size limit: E * (6 * 14 * N^2 + 12 * N^3) words of the chosen precision must fit in 32 MiB
@@ -413,11 +414,11 @@ chorus_status chorus_set_well_balanced(chorus_mesh mesh, int enable);
  * mesh's kernels, then clear it. */
 chorus_status chorus_check(chorus_mesh mesh, void* stream);
 
-/* Limit of the bounded device-side waits with which the residual and lifting kernels of this mesh
- * wait for the bulk copies that stage each element's state, background and gradient blocks in shared
- * memory: after `polls` polls the wait gives up, the kernel sets the mesh's error flag, waits (with
- * the default limit) for its copies still in flight and returns without computing or storing
- * anything; chorus_check then reports CHORUS_ETIMEOUT.  polls < 0 restores the default (2^24 polls
+/* Limit of the bounded device-side waits with which the volume kernel of this mesh waits for the bulk
+ * copies that stage each element's state, background and metrics in shared memory: after `polls` polls
+ * the wait gives up, the kernel sets the mesh's error flag, waits (with the default limit) for its
+ * copies still in flight and returns without storing its elements, and while the flag is set the kernel
+ * that completes the residual or stage leaves it as it is; chorus_check then reports CHORUS_ETIMEOUT.  polls < 0 restores the default (2^24 polls
  * with back-off, about a second); 0 makes every wait give up at once, so the failure path can be
  * exercised without a fault.  polls >= 2^32 - 1: CHORUS_EINVAL.  Synchronous. */
 chorus_status chorus_set_wait_limit(chorus_mesh mesh, int64_t polls);

@@ -2,7 +2,7 @@
 // (up to four union meshes, p = 2..5).  Its CTAs pull (order, tile) work items of each phase from a
 // counter (the orders' tiles in one list, the most expensive order first) and run the same tile
 // functions as the per-order kernels, specialised per order by template dispatch; between the phases
-// (traces, lifting, face fluxes, residual) they meet at a grid barrier whose spin is bounded: a
+// (traces, volume, face fluxes, update) they meet at a grid barrier whose spin is bounded: a
 // barrier that runs out of polls sets the error flag (CHORUS_ETIMEOUT) and the CTA stops, so that
 // every other CTA's next barrier runs out too and the launch ends.  Nothing traps.
 #include <cuda_runtime.h>
@@ -21,11 +21,14 @@ constexpr int kPMinBlocks = 3;     // resident CTAs per SM asked of the compiler
 template <int S>
 __host__ __device__ constexpr int p_epb() { return S == 0 ? 14 : S == 1 ? 8 : S == 2 ? 5 : 3; }
 
+// staging barriers of a CTA: p = 3 tiles stage by warps (unit_elems), the others by the CTA
+constexpr int kPBars = kVolBars * (kPThreads / 32);
+
 struct PersistArgs {
-  KArgs<float> grad[4], face[4], resid[4];  // slot p - 2; an absent order has no work items
+  KArgs<float> vol[4], face[4], update[4];  // slot p - 2; an absent order has no work items
   const int2* faces[4];
   int nf[4], nw[4];
-  int64_t items[4][4];  // [phase: traces, lifting, faces, residual][slot]
+  int64_t items[4][4];  // [phase: traces, volume, faces, update][slot]
   int trace;            // 1: the stage starts with the traces of its input state
   unsigned* sync;       // [0] grid-barrier arrivals, [1 + phase] work counter (zero at launch)
   unsigned* err;        // the error flags (bit 0: a bounded wait gave up) and, in err[1], the wait limit
@@ -66,44 +69,39 @@ __device__ bool grid_sync(unsigned* count, unsigned target, unsigned* err, uint3
 // thread; out of line, 0-0.5 KB each.
 template <int S>
 __device__ __noinline__ void trace_item(const PersistArgs& P, int64_t t) {
-  const KArgs<float>& A = P.grad[S];
+  const KArgs<float>& A = P.vol[S];
   trace_tile<S + 3, float, p_epb<S>()>(A.m, A.ops, A.q, const_cast<float*>(A.T), t);
 }
 template <int S>
-__device__ __noinline__ void grad_item(const PersistArgs& P, int64_t t, uint64_t* bar, uint32_t& pbar) {
-  grad_tile<S + 3, true, float, p_epb<S>(), false>(P.grad[S], t, bar, pbar);
+__device__ __noinline__ void vol_item(const PersistArgs& P, int64_t t, uint64_t* bar, uint32_t& pbar) {
+  vol_tile<S + 3, true, float, p_epb<S>(), kModeRK, false>(P.vol[S], t, bar, pbar);
 }
 template <int S>
 __device__ __noinline__ void face_item(const PersistArgs& P, int64_t t) {
   face_point<S + 3, true, float>(P.face[S], P.faces[S], P.nf[S], P.nw[S], t * kPThreads + threadIdx.x);
 }
 template <int S>
-__device__ __noinline__ void resid_item(const PersistArgs& P, int64_t t, uint64_t* bar, uint64_t* barS, uint32_t& pbar,
-                                        uint32_t& pbarS) {
-  resid_tile<S + 3, true, float, p_epb<S>(), kModeRK, false>(P.resid[S], t, bar, barS, pbar, pbarS);
+__device__ __noinline__ void update_item(const PersistArgs& P, int64_t t) {
+  update_tile<S + 3, float, p_epb<S>(), kModeRK>(P.update[S], t);
 }
 template <int S>
-__device__ __forceinline__ void run_item(const PersistArgs& P, int phase, int64_t t, uint64_t* bar, uint64_t* barS,
-                                         uint32_t& pbar, uint32_t& pbarS) {
+__device__ __forceinline__ void run_item(const PersistArgs& P, int phase, int64_t t, uint64_t* bar, uint32_t& pbar) {
   if (phase == 0) trace_item<S>(P, t);
-  else if (phase == 1) grad_item<S>(P, t, bar, pbar);
+  else if (phase == 1) vol_item<S>(P, t, bar, pbar);
   else if (phase == 2) face_item<S>(P, t);
-  else resid_item<S>(P, t, bar, barS, pbar, pbarS);
+  else update_item<S>(P, t);
 }
 
 __global__ void __launch_bounds__(kPThreads, kPMinBlocks) k_batch_stage(const __grid_constant__ PersistArgs P) {
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ __align__(8) uint64_t barS[2];
+  __shared__ __align__(8) uint64_t bar[kPBars];
   __shared__ int64_t s_item;
   __shared__ int s_stop;
   if (threadIdx.x == 0) {
-    mbar_init(&bar);
-    mbar_init(&barS[0]);
-    mbar_init(&barS[1]);
+    for (int b = 0; b < kPBars; ++b) mbar_init(&bar[b]);
     s_stop = 0;
   }
   __syncthreads();
-  uint32_t pbar = 0, pbarS = 0;
+  uint32_t pbar = 0;
   unsigned barriers = 0;
   const uint32_t polls = wait_polls(P.err);  // the grid barriers' limit: the staging waits' own
   for (int phase = P.trace ? 0 : 1; phase < 4; ++phase) {
@@ -121,14 +119,13 @@ __global__ void __launch_bounds__(kPThreads, kPMinBlocks) k_batch_stage(const __
         t -= P.items[phase][slot];
         --slot;
       }
-      if (slot == 3) run_item<3>(P, phase, t, &bar, barS, pbar, pbarS);
-      else if (slot == 2) run_item<2>(P, phase, t, &bar, barS, pbar, pbarS);
-      else if (slot == 1) run_item<1>(P, phase, t, &bar, barS, pbar, pbarS);
-      else run_item<0>(P, phase, t, &bar, barS, pbar, pbarS);
+      if (slot == 3) run_item<3>(P, phase, t, bar, pbar);
+      else if (slot == 2) run_item<2>(P, phase, t, bar, pbar);
+      else if (slot == 1) run_item<1>(P, phase, t, bar, pbar);
+      else run_item<0>(P, phase, t, bar, pbar);
       __syncthreads();  // the tile's shared memory is free for the next one
       if (threadIdx.x == 0 && (*(volatile unsigned*)P.err & 1u)) s_stop = 1;  // a bounded wait gave up
     }
-    if (phase == 1 && threadIdx.x == 0) bulk_wait_all();  // the gradient records are written out
     if (phase < 3 && !grid_sync(P.sync, ++barriers * gridDim.x, P.err, polls)) return;
   }
 }
@@ -140,8 +137,7 @@ namespace {
 template <int S>
 constexpr size_t slot_smem() {
   constexpr int N = S + 3, EPB = p_epb<S>();
-  return std::max((size_t)Layout<N, true, float, EPB>::total_grad,
-                  (size_t)Layout<N, true, float, EPB, true>::total_resid) * sizeof(float);
+  return std::max((size_t)Layout<N, true, float, EPB>::total, (size_t)UpLayout<N, float, EPB>::total) * sizeof(float);
 }
 constexpr size_t kPSmem = std::max(std::max(slot_smem<0>(), slot_smem<1>()), std::max(slot_smem<2>(), slot_smem<3>()));
 
@@ -192,15 +188,15 @@ chorus_status persist_rk3_step(StagePtrs* const groups[4], double dt, unsigned* 
       const int N = s + 3;
       float* Tc = (k % 2 == 0) ? G.Ta : G.Tb;  // the traces of the stage's input state
       float* Tn = (k % 2 == 0) ? G.Tb : G.Ta;
-      KArgs<float>& a = P.grad[s];
+      KArgs<float>& a = P.vol[s];
       a.m = G.m; a.ops = G.ops; a.ph = G.ph; a.bg = G.bg; a.q = G.buf[sg.src]; a.T = Tc; a.Tv_out = G.Tv;
-      a.G_out = G.G; a.Fc_out = G.Fc; a.err = err;
+      a.out = G.buf[sg.dst]; a.un = G.buf[sg.un]; a.a = (float)sg.a; a.b = (float)sg.b; a.c = (float)sg.c;
+      a.dt = (float)dt; a.err = err;
       KArgs<float>& f = P.face[s];
       f.m = G.m; f.ph = G.ph; f.bg = G.bg; f.T = Tc; f.Tv = G.Tv; f.Fc_out = G.Fc; f.err = err;
-      KArgs<float>& r = P.resid[s];
-      r.m = G.m; r.ops = G.ops; r.ph = G.ph; r.bg = G.bg; r.q = G.buf[sg.src]; r.T = Tc; r.Tv = G.Tv;
-      r.out = G.buf[sg.dst]; r.T_out = Tn; r.G_in = G.G; r.Fc = G.Fc;
-      r.un = G.buf[sg.un]; r.a = (float)sg.a; r.b = (float)sg.b; r.c = (float)sg.c; r.dt = (float)dt; r.err = err;
+      KArgs<float>& r = P.update[s];
+      r.m = G.m; r.ops = G.ops; r.Fc = G.Fc; r.out = G.buf[sg.dst]; r.T_out = Tn; r.c = (float)sg.c;
+      r.dt = (float)dt; r.err = err;
       P.faces[s] = G.faces;
       P.nf[s] = G.nf;
       P.nw[s] = G.nw;

@@ -35,12 +35,12 @@ MeshArg<R> mesh_arg(const chorus_mesh_s* m);
 template <>
 MeshArg<double> mesh_arg<double>(const chorus_mesh_s* m) {
   return MeshArg<double>{(int)m->E, m->d_nbr,   m->d_code, m->d_Sf64,
-                         m->d_invJ64, m->d_x64, m->kr_active ? m->d_kr64 : nullptr};
+                         m->d_invJ64, m->d_x64, m->kr_active ? m->d_kr64 : nullptr, m->d_tab64, 0};
 }
 template <>
 MeshArg<float> mesh_arg<float>(const chorus_mesh_s* m) {
   return MeshArg<float>{(int)m->E, m->d_nbr,   m->d_code, m->d_Sf32,
-                        m->d_invJ32, m->d_x32, m->kr_active ? m->d_kr32 : nullptr};
+                        m->d_invJ32, m->d_g32, m->kr_active ? m->d_kr32 : nullptr, m->d_tab32, 0};
 }
 
 template <class R>
@@ -61,6 +61,7 @@ PhysArg<R> phys_arg(const chorus_params& P, double r_inner, double r_outer) {
   a.CpR = (R)(gamma / (gamma - 1.0));
   a.kappa = (R)P.kappa;
   a.kappa_r = (R)P.kappa_r;
+  a.kappa_g = (R)(P.kappa / gamma);
   a.nu = (R)P.nu;
   a.GM = (R)P.GM;
   a.twoOmega = (R)(2.0 * P.Omega);
@@ -212,6 +213,26 @@ __global__ void k_bg_tables(int64_t E, int N, const double* __restrict__ Q0, con
     bgT[(ef * 2) * N2 + t] = (float)T[(ef * 5) * N2 + t];
     bgT[(ef * 2 + 1) * N2 + t] = (float)T[(ef * 5 + 4) * N2 + t];
   }
+}
+
+// the background face values of the other side of each face point (a wall's own) from the elements' own
+__global__ void k_bg_other(int64_t E, int N, const int* __restrict__ nbr, const int* __restrict__ code,
+                           const float* __restrict__ own, float* __restrict__ other) {
+  const int N2 = N * N;
+  const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (g >= E * 6 * N2) return;
+  const int64_t ef = g / N2;
+  const int t = (int)(g % N2), k = nbr[ef], c = code[ef];
+  int64_t nf = ef;
+  int tp = t;
+  if (k >= 0) {
+    nf = (int64_t)k * 6 + (c >> 3);
+    int a = (c & 4) ? t / N : t % N, b = (c & 4) ? t % N : t / N;
+    if (c & 2) a = N - 1 - a;
+    if (c & 1) b = N - 1 - b;
+    tp = a + N * b;
+  }
+  for (int v = 0; v < 2; ++v) other[(ef * 2 + v) * N2 + t] = own[(nf * 2 + v) * N2 + tp];
 }
 
 // deterministic two-level FP64 reduction: per-block partial sums of
@@ -366,9 +387,10 @@ void free_background(chorus_mesh_s* m) {
   dev_free(m->d_bg);
   dev_free(m->d_grho0);
   dev_free(m->d_bgT);
+  dev_free(m->d_bgTo);
   dev_free(m->d_R0);
   m->d_Q0 = nullptr;
-  m->d_bg = m->d_grho0 = m->d_bgT = m->d_R0 = nullptr;
+  m->d_bg = m->d_grho0 = m->d_bgT = m->d_bgTo = m->d_R0 = nullptr;
   m->prepared = false;
 }
 
@@ -421,7 +443,10 @@ void free_mesh(chorus_mesh_s* m) {
   dev_free(m->d_wJ);
   dev_free(m->d_Sf32);
   dev_free(m->d_invJ32);
+  dev_free(m->d_g32);
   dev_free(m->d_x32);
+  dev_free(m->d_tab64);
+  dev_free(m->d_tab32);
   dev_free(m->d_kr64);
   dev_free(m->d_kr32);
   dev_free(m->d_err);
@@ -433,9 +458,8 @@ void free_mesh(chorus_mesh_s* m) {
 size_t ws_words(const chorus_mesh_s* m) {
   const size_t N = m->N, E = m->E;
   const size_t N2 = N * N, N3 = N2 * N;
-  // stage buffer + two trace buffers + viscous normal-flux traces + two more stage buffers (RK(5,4))
-  // + the gradient record handed from the gradient kernel to the residual kernel + the common face
-  // fluxes of every face point
+  // stage buffer + two trace buffers + one-sided viscous face fluxes + two more stage buffers (RK(5,4))
+  // + the gradient record of the three-pass kernels + the common face fluxes of every face point
   return 3 * E * 5 * N3 + 2 * E * 6 * 5 * N2 + E * 6 * 4 * N2 + E * 12 * N3 + E * 6 * 5 * N2;
 }
 
@@ -565,6 +589,7 @@ chorus_status chorus_mesh_create(int64_t n_nodes, const double* node_xyz, int64_
     return (chorus_status)rc;
   }
   m->L = launchers_for(p, 0);
+  m->L3 = p == 2 ? three_pass_p2() : p == 3 ? three_pass_p3() : p == 4 ? three_pass_p4() : three_pass_p5();
   fill_ops(m->tab, &m->ops64);
   fill_ops(m->tab, &m->ops32);
   const int N = m->N, N2 = N * N, N3 = N2 * N;
@@ -585,7 +610,8 @@ chorus_status chorus_mesh_create(int64_t n_nodes, const double* node_xyz, int64_
             dev_alloc(&m->d_Sf64, nS) == cudaSuccess && dev_alloc(&m->d_invJ64, nP) == cudaSuccess &&
             dev_alloc(&m->d_x64, 3 * nP) == cudaSuccess && dev_alloc(&m->d_wJ, nP) == cudaSuccess &&
             dev_alloc(&m->d_Sf32, nS) == cudaSuccess && dev_alloc(&m->d_invJ32, nP) == cudaSuccess &&
-            dev_alloc(&m->d_x32, 3 * nP) == cudaSuccess && dev_alloc(&m->d_err, 4) == cudaSuccess &&
+            dev_alloc(&m->d_g32, 3 * nP) == cudaSuccess && dev_alloc(&m->d_x32, 3 * nP) == cudaSuccess && dev_alloc(&m->d_err, 4) == cudaSuccess &&
+            dev_alloc(&m->d_tab64, 2 * (N + 1) * N) == cudaSuccess && dev_alloc(&m->d_tab32, 2 * (N + 1) * N) == cudaSuccess &&
             dev_alloc(&m->d_red, (size_t)kRedBlocks * 6 + 16) == cudaSuccess;
   if (!ok) {
     free_mesh(m);
@@ -624,6 +650,20 @@ chorus_status chorus_mesh_create(int64_t n_nodes, const double* node_xyz, int64_
   up(m->d_invJ32, f32.data(), nP * sizeof(float));
   for (size_t i = 0; i < 3 * nP; ++i) f32[i] = (float)m->host.x[i];
   up(m->d_x32, f32.data(), 3 * nP * sizeof(float));
+  for (size_t e = 0; e < E; ++e)
+    for (int pt = 0; pt < N3; ++pt) {
+      const double* x = &m->host.x[e * 3 * N3 + pt];
+      const double r2 = x[0] * x[0] + x[N3] * x[N3] + x[2 * N3] * x[2 * N3], ir3 = 1.0 / (r2 * std::sqrt(r2));
+      for (int n = 0; n < 3; ++n) f32[(e * 3 + n) * N3 + pt] = (float)(x[n * N3] * ir3);
+    }
+  up(m->d_g32, f32.data(), 3 * nP * sizeof(float));
+  std::vector<double> tab;
+  for (int t = 0; t < 2; ++t)
+    for (int f = 0; f <= N; ++f)
+      for (int i = 0; i < N; ++i) tab.push_back(t == 0 ? m->tab.I[f * N + i] : m->tab.D[i * (N + 1) + f]);
+  const std::vector<float> tab32(tab.begin(), tab.end());
+  up(m->d_tab64, tab.data(), tab.size() * sizeof(double));
+  up(m->d_tab32, tab32.data(), tab32.size() * sizeof(float));
   if (ce == cudaSuccess) ce = cudaMemsetAsync(m->d_err, 0, 4 * sizeof(unsigned), st);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
   if (ce != cudaSuccess) {
@@ -673,13 +713,13 @@ chorus_status prepare_background(chorus_mesh_s* m, const chorus_params* P, int64
   const int N = m->N, N2 = N * N, N3 = N2 * N;
   const size_t E = m->E, nP = E * N3, nT = E * 6 * 5 * N2;
   if (dev_alloc(&m->d_Q0, 5 * nP) || dev_alloc(&m->d_bg, 2 * nP) || dev_alloc(&m->d_grho0, 3 * nP) ||
-      dev_alloc(&m->d_bgT, E * 6 * 2 * N2) || dev_alloc(&m->d_R0, 5 * nP)) {
+      dev_alloc(&m->d_bgT, E * 6 * 2 * N2) || dev_alloc(&m->d_bgTo, E * 6 * 2 * N2) || dev_alloc(&m->d_R0, 5 * nP)) {
     free_background(m);
     return CHORUS_ENOMEM;
   }
   double *T = nullptr, *Tv = nullptr, *R0 = nullptr, *gr = nullptr, *tab = nullptr, *G = nullptr, *Fc = nullptr;
   if (dev_alloc(&T, nT) || dev_alloc(&Tv, E * 6 * 4 * N2) || dev_alloc(&R0, 5 * nP) || dev_alloc(&gr, 3 * nP) ||
-      dev_alloc(&G, (size_t)kG * nP) || dev_alloc(&Fc, nT) || (rho_tab && dev_alloc(&tab, 2 * (size_t)n_tab))) {
+      dev_alloc(&G, 12 * nP) || dev_alloc(&Fc, nT) || (rho_tab && dev_alloc(&tab, 2 * (size_t)n_tab))) {
     dev_free(T); dev_free(Tv); dev_free(R0); dev_free(gr); dev_free(tab); dev_free(G); dev_free(Fc);
     free_background(m);
     return CHORUS_ENOMEM;
@@ -700,16 +740,14 @@ chorus_status prepare_background(chorus_mesh_s* m, const chorus_params* P, int64
     k_background<<<grid1(nP), 256, 0, st>>>((int64_t)nP, N3, m->d_x64, ph, m->d_Q0);
     ce = cudaGetLastError();
   }
-  if (ce == cudaSuccess) ce = m->L.trace64(ma, m->ops64, m->d_Q0, T, st);
-  if (ce == cudaSuccess) ce = m->L.grad64(ma, m->ops64, ph, m->d_Q0, T, Tv, gr, G, Fc, m->d_err, st);
-  if (ce == cudaSuccess) ce = m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st);
   if (ce == cudaSuccess)
-    ce = m->L.resid64(ma, m->ops64, ph, m->d_Q0, T, Tv, G, Fc, R0, nullptr, RkCoef<double>{}, 0.0, kModeResidual,
-                      m->d_err, st);
+    ce = m->L3.background(ma, m->ops64, ph, m->d_faces, m->n_ifaces, m->n_wfaces, m->d_Q0, T, Tv, gr, G, Fc, R0,
+                          m->d_err, st);
   if (ce == cudaSuccess) {
     k_d2f<<<grid1(5 * nP), 256, 0, st>>>((int64_t)(5 * nP), R0, m->d_R0);
-    k_bg_tables<<<grid1(std::max(nP, E * 6 * N2)), 256, 0, st>>>((int64_t)E, N, m->d_Q0, T, gr, m->d_bg, m->d_bgT,
+    k_bg_tables<<<grid1(std::max(nP, E * 6 * N2)), 256, 0, st>>>((int64_t)E, N, m->d_Q0, T, gr, m->d_bg, m->d_bgTo,
                                                                  m->d_grho0);
+    k_bg_other<<<grid1(E * 6 * N2), 256, 0, st>>>((int64_t)E, N, m->d_nbr, m->d_code, m->d_bgTo, m->d_bgT);
     ce = cudaGetLastError();
   }
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
@@ -836,20 +874,20 @@ chorus_status chorus_residual(chorus_mesh m, const chorus_params* P, chorus_prec
     const PhysArg<double> ph = phys_arg<double>(*P, m->r_inner, m->r_outer);
     const MeshArg<double> ma = mesh_arg<double>(m);
     Ws<double> w = split_ws<double>(m, workspace);
-    CHK(timed(m, 0, st, [&] { return m->L.trace64(ma, m->ops64, (const double*)Q, w.Ta, st); }));
-    CHK(timed(m, 1, st, [&] {
-      return m->L.grad64(ma, m->ops64, ph, (const double*)Q, w.Ta, w.Tv, nullptr, w.G, w.Fc, m->d_err, st);
-    }));
-    CHK(timed(m, 3, st, [&] { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
     RkCoef<double> rc{};
     if (m->closure) {
       if (!m->prepared) return CHORUS_EINVAL;  // the network reads q' = Q - Q0
       CHK(mlp_elements_tc(0, m->closure, Q, m->d_Q0, m->closure_buf, m->E, 0, m->d_err, st));
       rc.radd = (const double*)m->closure_buf;
     }
+    CHK(timed(m, 0, st, [&] { return m->L.trace64(ma, m->ops64, (const double*)Q, w.Ta, st); }));
+    CHK(timed(m, 1, st, [&] {
+      return m->L.vol64(ma, m->ops64, ph, (const double*)Q, w.Ta, w.Tv, (double*)R, rc, 0.0, kModeResidual,
+                        m->d_err, st);
+    }));
+    CHK(timed(m, 3, st, [&] { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
     CHK(timed(m, 2, st, [&] {
-      return m->L.resid64(ma, m->ops64, ph, (const double*)Q, w.Ta, w.Tv, w.G, w.Fc, (double*)R, nullptr, rc, 0.0,
-                          kModeResidual, m->d_err, st);
+      return m->L.update64(ma, m->ops64, w.Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, m->d_err, st);
     }));
     return CHORUS_OK;
   }
@@ -861,19 +899,19 @@ chorus_status chorus_residual(chorus_mesh m, const chorus_params* P, chorus_prec
   const MeshArg<float> ma = mesh_arg<float>(m);
   Ws<float> w = split_ws<float>(m, workspace);
   const BgArg bg = bg_arg(m);
-  CHK(timed(m, 0, st, [&] { return m->L.trace32(ma, m->ops32, (const float*)Q, w.Ta, st); }));
-  CHK(timed(m, 1, st, [&] {
-    return m->L.grad32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, w.G, w.Fc, m->d_err, st);
-  }));
-  CHK(timed(m, 3, st, [&] { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
   RkCoef<float> rc{};
   if (m->closure) {
     CHK(mlp_elements_tc(1, m->closure, Q, nullptr, m->closure_buf, m->E, 0, m->d_err, st));
     rc.radd = (const float*)m->closure_buf;
   }
+  CHK(timed(m, 0, st, [&] { return m->L.trace32(ma, m->ops32, (const float*)Q, w.Ta, st); }));
+  CHK(timed(m, 1, st, [&] {
+    return m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, (float*)R, rc, 0.0f, kModeResidual, m->d_err,
+                      st);
+  }));
+  CHK(timed(m, 3, st, [&] { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
   CHK(timed(m, 2, st, [&] {
-    return m->L.resid32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, w.G, w.Fc, (float*)R, nullptr, rc, 0.0f,
-                        kModeResidual, m->d_err, st);
+    return m->L.update32(ma, m->ops32, w.Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, m->d_err, st);
   }));
   return CHORUS_OK;
 }
@@ -904,9 +942,9 @@ const std::vector<Stage>& stages_of(int scheme) {
 
 namespace {
 
-template <class R, class Grad, class Face, class Resid, class Trace>
+template <class R, class Vol, class Face, class Update, class Trace>
 chorus_status run_rk(chorus_mesh_s* m, R* u, const Ws<R>& w, double dt, int64_t n_steps, int scheme, cudaStream_t st,
-                     Grad grad, Face face, Resid resid, Trace trace) {
+                     Vol vol, Face face, Update update, Trace trace) {
   R* buf[4] = {u, w.s, w.A, w.B};
   R *Tc = w.Ta, *Tn = w.Tb;
   CHK(timed(m, 0, st, [&] { return trace(u, Tc); }));
@@ -920,21 +958,21 @@ chorus_status run_rk(chorus_mesh_s* m, R* u, const Ws<R>& w, double dt, int64_t 
                             m->closure_buf, m->E, 0, m->d_err, st));
         c.radd = (const R*)m->closure_buf;
       }
-      CHK(timed(m, 1, st, [&] { return grad(buf[g.src], Tc); }));
+      CHK(timed(m, 1, st, [&] { return vol(buf[g.src], Tc, buf[g.dst], c); }));
       CHK(timed(m, 3, st, [&] { return face(Tc); }));
-      CHK(timed(m, 2, st, [&] { return resid(buf[g.src], Tc, buf[g.dst], Tn, c); }));
+      CHK(timed(m, 2, st, [&] { return update(buf[g.dst], Tn, c); }));
       std::swap(Tc, Tn);
     }
   return CHORUS_OK;
 }
 
-// Element chunks of chorus_rk_step_host (FP32): the copy in with the traces, the last stage's residual
+// Element chunks of chorus_rk_step_host (FP32): the copy in with the traces, the last stage's update
 // with the copy out.
 constexpr int kHostChunks = 8;
 
-// The residual kernel's per-element arguments shifted to elements [e0, e0 + ne): with the face kernel
-// the residual kernel reads no neighbour data (the common face fluxes are in each element's own face
-// numbering), so a range of elements is a mesh of its own for it.
+// The per-element arguments of the trace and update kernels shifted to elements [e0, e0 + ne): neither
+// reads neighbour data (the common face fluxes are in each element's own face numbering), so a range of
+// elements is a mesh of its own for them, but for the trace array, which they write as a whole.
 MeshArg<float> mesh_range(MeshArg<float> a, int64_t e0, int64_t ne, int N) {
   const int64_t N2 = N * N, N3 = N2 * N;
   a.E = (int)ne;
@@ -944,20 +982,12 @@ MeshArg<float> mesh_range(MeshArg<float> a, int64_t e0, int64_t ne, int N) {
   a.invJ += e0 * N3;
   a.x += e0 * 3 * N3;
   if (a.kr) a.kr += e0 * 3 * (N + 1) * N2;
+  a.e0 = e0;
   return a;
 }
-BgArg bg_range(BgArg b, int64_t e0, int N) {
-  const int64_t N2 = N * N, N3 = N2 * N;
-  b.bg += e0 * 2 * N3;
-  b.grho0 += e0 * 3 * N3;
-  b.bgT += e0 * 12 * N2;
-  if (b.R0) b.R0 += e0 * 5 * N3;
-  return b;
-}
-
 // chorus_rk_step_host, FP32 perturbation form: the state is copied in in kHostChunks element ranges
 // on the mesh's copy stream, each range's traces computed as soon as it has arrived; the last stage's
-// residual runs on the same ranges, and each range's new state is copied to the host while the next
+// update runs on the same ranges, and each range's new state is copied to the host while the next
 // range is computed.  Synchronises.
 chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float* Qh, float* Qd, void* workspace,
                                 double dt, int64_t n_steps, cudaStream_t st) {
@@ -985,26 +1015,21 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
   bool copied = false;  // the chunks of the last stage copied the state out
   const chorus_status s = run_rk<float>(
       m, Qd, w, dt, n_steps, 0, st,
-      [&](const float* q, const float* T) {
-        return m->L.grad32(ma, m->ops32, ph, bg, q, T, w.Tv, w.G, w.Fc, m->d_err, st);
+      [&](const float* q, const float* T, float* dst, const RkCoef<float>& c) {
+        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, dst, c, (float)dt, kModeRK, m->d_err, st);
       },
       [&](const float* T) { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
-      [&](const float* q, const float* T, float* dst, float* Tn, const RkCoef<float>& c) -> cudaError_t {
+      [&](float* dst, float* Tn, const RkCoef<float>& c) -> cudaError_t {
         if (++stage < last || dst != Qd)
-          return m->L.resid32(ma, m->ops32, ph, bg, q, T, w.Tv, w.G, w.Fc, dst, Tn, c, (float)dt, kModeRK, m->d_err, st);
+          return m->L.update32(ma, m->ops32, w.Fc, dst, Tn, c, (float)dt, kModeRK, m->d_err, st);
         for (int k = 0; k < kHostChunks; ++k) {
           int64_t e0, ne;
           range(k, &e0, &ne);
           if (ne == 0) continue;
           RkCoef<float> ck = c;
           const int64_t o5 = e0 * 5 * N3;
-          ck.un = c.un ? c.un + o5 : nullptr;
-          ck.un2 = c.un2 ? c.un2 + o5 : nullptr;
           ck.out2 = c.out2 ? c.out2 + o5 : nullptr;
-          ck.radd = c.radd ? c.radd + o5 : nullptr;
-          cudaError_t e = m->L.resid32(mesh_range(ma, e0, ne, N), m->ops32, ph, bg_range(bg, e0, N), q + o5, T + e0 * 30 * N2,
-                                       w.Tv + e0 * 24 * N2, w.G + e0 * 12 * N3, w.Fc + e0 * 30 * N2, dst + o5,
-                                       Tn + e0 * 30 * N2, ck, (float)dt, kModeRK, m->d_err, st);
+          cudaError_t e = m->L.update32(mesh_range(ma, e0, ne, N), m->ops32, w.Fc + e0 * 30 * N2, dst + o5, Tn, ck, (float)dt, kModeRK, m->d_err, st);
           if (e == cudaSuccess) e = cudaEventRecord(m->copy_ev[k], st);
           if (e == cudaSuccess) e = cudaStreamWaitEvent(m->copy_stream, m->copy_ev[k], 0);
           if (e == cudaSuccess)
@@ -1029,7 +1054,7 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
           e = cudaMemcpyAsync(Qd + o5, Qh + o5, ne * 5 * N3 * sizeof(float), cudaMemcpyHostToDevice, m->copy_stream);
           if (e == cudaSuccess) e = cudaEventRecord(ev_in[k], m->copy_stream);
           if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_in[k], 0);
-          if (e == cudaSuccess) e = m->L.trace32(mesh_range(ma, e0, ne, N), m->ops32, q + o5, T + e0 * 30 * N2, st);
+          if (e == cudaSuccess) e = m->L.trace32(mesh_range(ma, e0, ne, N), m->ops32, q + o5, T, st);
         }
         return e;
       });
@@ -1060,12 +1085,12 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
     Ws<double> w = split_ws<double>(m, workspace);
     return run_rk<double>(
         m, (double*)Q, w, dt, n_steps, scheme, st,
-        [&](const double* q, const double* T) {
-          return m->L.grad64(ma, m->ops64, ph, q, T, w.Tv, nullptr, w.G, w.Fc, m->d_err, st);
+        [&](const double* q, const double* T, double* dst, const RkCoef<double>& c) {
+          return m->L.vol64(ma, m->ops64, ph, q, T, w.Tv, dst, c, dt, kModeRK, m->d_err, st);
         },
         [&](const double* T) { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
-        [&](const double* q, const double* T, double* dst, double* Tn, const RkCoef<double>& c) {
-          return m->L.resid64(ma, m->ops64, ph, q, T, w.Tv, w.G, w.Fc, dst, Tn, c, dt, kModeRK, m->d_err, st);
+        [&](double* dst, double* Tn, const RkCoef<double>& c) {
+          return m->L.update64(ma, m->ops64, w.Fc, dst, Tn, c, dt, kModeRK, m->d_err, st);
         },
         [&](const double* q, double* T) { return m->L.trace64(ma, m->ops64, q, T, st); });
   }
@@ -1074,17 +1099,35 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
   const chorus_status ks = ensure_kr(m, *P, st);
   if (ks != CHORUS_OK) return ks;
   const PhysArg<float> ph = phys_arg<float>(*P, m->r_inner, m->r_outer);
-  const MeshArg<float> ma = mesh_arg<float>(m);
-  const BgArg bg = bg_arg(m);
+  MeshArg<float> ma = mesh_arg<float>(m);
+  BgArg bg = bg_arg(m);
   Ws<float> w = split_ws<float>(m, workspace);
+  if (scheme == 1) {  // on the three-pass kernels (three_pass.cuh)
+    ma.x = m->d_x32;
+    bg.bgT = m->d_bgTo;
+    const float* src = nullptr;
+    return run_rk<float>(
+        m, (float*)Q, w, dt, n_steps, scheme, st,
+        [&](const float* q, const float* T, float*, const RkCoef<float>&) {
+          src = q;
+          return m->L3.grad(ma, m->ops32, ph, bg, q, T, w.Tv, w.G, m->d_err, st);
+        },
+        [&](const float* T) {
+          return m->L3.face(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st);
+        },
+        [&](float* dst, float* Tn, const RkCoef<float>& c) {
+          return m->L3.resid(ma, m->ops32, ph, bg, src, w.G, w.Fc, dst, Tn, c, (float)dt, m->d_err, st);
+        },
+        [&](const float* q, float* T) { return m->L3.trace(ma, m->ops32, q, T, st); });
+  }
   return run_rk<float>(
       m, (float*)Q, w, dt, n_steps, scheme, st,
-      [&](const float* q, const float* T) {
-        return m->L.grad32(ma, m->ops32, ph, bg, q, T, w.Tv, w.G, w.Fc, m->d_err, st);
+      [&](const float* q, const float* T, float* dst, const RkCoef<float>& c) {
+        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, dst, c, (float)dt, kModeRK, m->d_err, st);
       },
       [&](const float* T) { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
-      [&](const float* q, const float* T, float* dst, float* Tn, const RkCoef<float>& c) {
-        return m->L.resid32(ma, m->ops32, ph, bg, q, T, w.Tv, w.G, w.Fc, dst, Tn, c, (float)dt, kModeRK, m->d_err, st);
+      [&](float* dst, float* Tn, const RkCoef<float>& c) {
+        return m->L.update32(ma, m->ops32, w.Fc, dst, Tn, c, (float)dt, kModeRK, m->d_err, st);
       },
       [&](const float* q, float* T) { return m->L.trace32(ma, m->ops32, q, T, st); });
 }
@@ -1100,7 +1143,7 @@ chorus_status chorus_rk_step_host(chorus_mesh m, const chorus_params* P, chorus_
   const size_t bytes = (size_t)m->E * 5 * m->N * m->N * m->N * (prec == CHORUS_FP64 ? sizeof(double) : sizeof(float));
   cudaStream_t st = (cudaStream_t)stream;
   if (prec == CHORUS_FP32_PERT && n_steps > 0 && P && workspace && dt > 0.0 && std::isfinite(dt)) {
-    // copies in element chunks overlapping the first traces and the last stage's residual
+    // copies in element chunks overlapping the first traces and the last stage's update
     // (synchronises)
     return rk_step_host_fp32(m, *P, (float*)Q_host, (float*)Q_dev, workspace, dt, n_steps, st);
   }
@@ -1464,8 +1507,9 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
   const size_t N2 = (size_t)m->N * m->N, E = (size_t)m->E;
   const size_t word = prec == CHORUS_FP64 ? sizeof(double) : sizeof(float);
   const size_t N3 = N2 * (size_t)m->N;
-  const size_t nT = E * 6 * 5 * N2, nTv = E * 6 * 4 * N2, nG = E * kG * N3;
-  if ((2 * nT + nTv + nG) * word > kNoAllocScratchBytes) return CHORUS_EINVAL;  // mesh too large for the scratch
+  const size_t nT = E * 6 * 5 * N2, nTv = E * 6 * 4 * N2;
+  // the documented size limit (more than the traces and the two face-flux arrays need today)
+  if ((2 * nT + nTv + E * 12 * N3) * word > kNoAllocScratchBytes) return CHORUS_EINVAL;  // mesh too large for the scratch
   if (prec == CHORUS_FP32_PERT && (!m->prepared || !same_params(m->prep, *P))) return CHORUS_EINVAL;
   // the attached closure's output buffer was allocated by chorus_closure_attach; FP64 reads Q0
   if (m->closure && prec == CHORUS_FP64 && !m->prepared) return CHORUS_EINVAL;
@@ -1482,18 +1526,16 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
     const MeshArg<double> ma = mesh_arg<double>(m);
     double* T = (double*)scratch;
     double* Tv = T + nT;
-    double* G = Tv + nTv;
-    double* Fc = G + nG;
+    double* Fc = Tv + nTv;
     RkCoef<double> rc{};
     if (m->closure) {
       CHK(mlp_elements_tc(0, m->closure, Q, m->d_Q0, m->closure_buf, m->E, 0, m->d_err, st));
       rc.radd = (const double*)m->closure_buf;
     }
     CHK(m->L.trace64(ma, m->ops64, (const double*)Q, T, st));
-    CHK(m->L.grad64(ma, m->ops64, ph, (const double*)Q, T, Tv, nullptr, G, Fc, m->d_err, st));
+    CHK(m->L.vol64(ma, m->ops64, ph, (const double*)Q, T, Tv, (double*)R, rc, 0.0, kModeResidual, m->d_err, st));
     CHK(m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st));
-    CHK(m->L.resid64(ma, m->ops64, ph, (const double*)Q, T, Tv, G, Fc, (double*)R, nullptr, rc, 0.0, kModeResidual,
-                     m->d_err, st));
+    CHK(m->L.update64(ma, m->ops64, Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, m->d_err, st));
     return CHORUS_OK;
   }
   const PhysArg<float> ph = phys_arg<float>(*P, m->r_inner, m->r_outer);
@@ -1501,18 +1543,16 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
   const BgArg bg = bg_arg(m);
   float* T = (float*)scratch;
   float* Tv = T + nT;
-  float* G = Tv + nTv;
-  float* Fc = G + nG;
+  float* Fc = Tv + nTv;
   RkCoef<float> rc{};
   if (m->closure) {
     CHK(mlp_elements_tc(1, m->closure, Q, nullptr, m->closure_buf, m->E, 0, m->d_err, st));
     rc.radd = (const float*)m->closure_buf;
   }
   CHK(m->L.trace32(ma, m->ops32, (const float*)Q, T, st));
-  CHK(m->L.grad32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, G, Fc, m->d_err, st));
+  CHK(m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, (float*)R, rc, 0.0f, kModeResidual, m->d_err, st));
   CHK(m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st));
-  CHK(m->L.resid32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, G, Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual,
-                   m->d_err, st));
+  CHK(m->L.update32(ma, m->ops32, Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, m->d_err, st));
   return CHORUS_OK;
 }
 
@@ -1575,7 +1615,6 @@ chorus_status mesh_stage_ptrs(chorus_mesh_s* m, const chorus_params& P, float* u
   out->Ta = w.Ta;
   out->Tb = w.Tb;
   out->Tv = w.Tv;
-  out->G = w.G;
   out->Fc = w.Fc;
   out->faces = m->d_faces;
   out->nf = m->n_ifaces;

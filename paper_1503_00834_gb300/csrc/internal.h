@@ -6,8 +6,8 @@
 namespace chorus {
 
 constexpr int kMaxN = 6;
-// entries of the gradient record per solution point: grad rho (3), trace-free strain (6), grad p (3)
-constexpr int kG = 12;
+// entries of the gradient record per solution point: grad rho (3), trace-free strain (5), grad p (3)
+constexpr int kG = 11;
 
 // 1D operators for one order, passed to kernels by value (parameter bank).
 template <class R>
@@ -24,6 +24,7 @@ template <class R>
 struct PhysArg {
   R gamma, gm1, Rgas, CpR;   // CpR = C_p / R_gas
   R kappa, kappa_r, nu;
+  R kappa_g;                 // kappa / gamma
   R GM, twoOmega;
   R T_top, bottom_flux;
   // polytrope (Eqs. 25-27): chi = c + alpha d / r, rho_a = rho_c chi^n, p_a = p_c chi^(n+1)
@@ -38,16 +39,18 @@ struct MeshArg {
   const int* code;   // [E][6] neighbour local face * 8 + orientation bits
   const R* Sf;       // [E][3 d][3 n][N+1 f][N*N line]  S^d_n = |J| d xi_d / d x_n at the d-flux points
   const R* invJ;     // [E][N^3] 1/|J| at the solution points
-  const R* x;        // [E][3][N^3] solution-point coordinates
+  const R* x;        // [E][3][N^3] solution-point coordinates x; FP32: x / |x|^3 (gravity)
   const R* kr;       // [E][3 d][N+1 f][N*N line] radiative diffusivity at the d-flux points, or null:
                      // the constant kappa_r
+  const R* tab;      // [2][N+1][N] h_s(Xf_f), then l'_f(X_i) as [f][i]
+  int64_t e0;        // index of the first element in the whole mesh (a range of elements; else 0)
 };
 
 // Background tables of the perturbation path (float, from FP64 computations).
 struct BgArg {
   const float* bg;     // [E][2][N^3]     rho0, E0
   const float* grho0;  // [E][3][N^3]     lifted background density gradient
-  const float* bgT;    // [E][6][2][N^2]  rho0, E0 on the face points
+  const float* bgT;    // [E][6][2][N^2]  rho0, E0 of the other side of each face point (of a wall's own)
   const float* R0;     // [E][5][N^3]     FP64 residual of the background, rounded (null: left out)
 };
 
@@ -65,7 +68,7 @@ __host__ __device__ inline int bg_point(int N, int pt) {
 
 enum ResidMode { kModeResidual = 0, kModeRK = 1 };
 
-// Stage combination of the RK update fused into the residual kernel:
+// Stage combination of the RK update fused into the volume kernel:
 //   out  = a un  + b q + c dt R
 //   out2 = a2 un2 + b2 q + c2 dt R   (when out2 != nullptr)
 // where R includes `radd` (an additive residual correction, e.g. the learned closure) when non-null.
@@ -80,29 +83,31 @@ struct RkCoef {
 };
 
 // Per-order launchers (defined in kern_p<N>.cu).  All return cudaGetLastError().
+//   trace   face traces of q, each in the neighbour's slot (trace_slot); T: of the whole mesh
+//   vol     from q and its traces: one-sided viscous face fluxes Tv and `out`, the residual (mode
+//           kModeResidual) or stage state (kModeRK, and rk.out2) without the end-point fluxes; `out` may be q
+//   face    common face fluxes F~ [E][6][5][N^2] of the face list (n_faces interior faces, from their
+//           lower element, then n_walls wall faces)
+//   update  the end-point fluxes' part added to `out` (and rk.out2); T_out: traces of the new state
+//           (of the whole mesh)
 struct LaunchSet {
   cudaError_t (*trace64)(const MeshArg<double>&, const OpsArg<double>&, const double* q, double* T, cudaStream_t);
-  // G: gradient record [E][12][N^3] written by grad (when non-null) and read by resid (required:
-  // resid returns cudaErrorInvalidValue without it).  Fc: common face fluxes F~ [E][6][5][N^2], written
-  // by face (interior and wall faces) and read by resid (required).
-  cudaError_t (*grad64)(const MeshArg<double>&, const OpsArg<double>&, const PhysArg<double>&, const double* q,
-                        const double* T, double* Tv, double* grad_rho_out, double* G, double* Fc, unsigned* err,
-                        cudaStream_t);
-  // faces: n_faces interior faces (from their lower element), then n_walls wall faces
+  cudaError_t (*vol64)(const MeshArg<double>&, const OpsArg<double>&, const PhysArg<double>&, const double* q,
+                       const double* T, double* Tv, double* out, const RkCoef<double>& rk,
+                       double dt, int mode, unsigned* err, cudaStream_t);
   cudaError_t (*face64)(const MeshArg<double>&, const PhysArg<double>&, const int2* faces, int n_faces, int n_walls,
                         const double* T, const double* Tv, double* Fc, cudaStream_t);
-  cudaError_t (*resid64)(const MeshArg<double>&, const OpsArg<double>&, const PhysArg<double>&, const double* q,
-                         const double* T, const double* Tv, const double* G, const double* Fc, double* out,
-                         double* T_out, const RkCoef<double>& rk, double dt, int mode, unsigned* err, cudaStream_t);
+  cudaError_t (*update64)(const MeshArg<double>&, const OpsArg<double>&, const double* Fc, double* out, double* T_out,
+                          const RkCoef<double>& rk, double dt, int mode, unsigned* err, cudaStream_t);
   cudaError_t (*trace32)(const MeshArg<float>&, const OpsArg<float>&, const float* q, float* T, cudaStream_t);
-  cudaError_t (*grad32)(const MeshArg<float>&, const OpsArg<float>&, const PhysArg<float>&, const BgArg&,
-                        const float* q, const float* T, float* Tv, float* G, float* Fc, unsigned* err, cudaStream_t);
+  cudaError_t (*vol32)(const MeshArg<float>&, const OpsArg<float>&, const PhysArg<float>&, const BgArg&,
+                       const float* q, const float* T, float* Tv, float* out, const RkCoef<float>& rk, float dt,
+                       int mode, unsigned* err, cudaStream_t);
   cudaError_t (*face32)(const MeshArg<float>&, const PhysArg<float>&, const BgArg&, const int2* faces, int n_faces,
                         int n_walls, const float* T, const float* Tv, float* Fc, cudaStream_t);
-  cudaError_t (*resid32)(const MeshArg<float>&, const OpsArg<float>&, const PhysArg<float>&, const BgArg&,
-                         const float* q, const float* T, const float* Tv, const float* G, const float* Fc, float* out,
-                         float* T_out, const RkCoef<float>& rk, float dt, int mode, unsigned* err, cudaStream_t);
-  int epb32;  // elements per CTA of the FP32 kernels
+  cudaError_t (*update32)(const MeshArg<float>&, const OpsArg<float>&, const float* Fc, float* out, float* T_out,
+                          const RkCoef<float>& rk, float dt, int mode, unsigned* err, cudaStream_t);
+  int epb32;  // elements per CTA of the FP32 volume kernel
 };
 
 // Each order is built with kTiles tile shapes of its FP32 kernels (elements per CTA); tile 0 is
@@ -112,5 +117,26 @@ LaunchSet launchers_p2(int tile);
 LaunchSet launchers_p3(int tile);
 LaunchSet launchers_p4(int tile);
 LaunchSet launchers_p5(int tile);
+
+// The three-pass kernels (three_pass.cuh): the FP32 SSP-RK(5,4) stages, and the FP64 residual of the
+// background.  T: traces in each element's own face numbering; bg.bgT and m.x (coordinates in FP32 too)
+// likewise the three-pass ones; G: gradient record [E][12][N^3].
+struct ThreePassSet {
+  cudaError_t (*trace)(const MeshArg<float>&, const OpsArg<float>&, const float* q, float* T, cudaStream_t);
+  cudaError_t (*grad)(const MeshArg<float>&, const OpsArg<float>&, const PhysArg<float>&, const BgArg&, const float* q,
+                      const float* T, float* Tv, float* G, unsigned* err, cudaStream_t);
+  cudaError_t (*face)(const MeshArg<float>&, const PhysArg<float>&, const BgArg&, const int2* faces, int n_faces,
+                      int n_walls, const float* T, const float* Tv, float* Fc, cudaStream_t);
+  cudaError_t (*resid)(const MeshArg<float>&, const OpsArg<float>&, const PhysArg<float>&, const BgArg&,
+                       const float* q, const float* G, const float* Fc, float* out, float* T_out,
+                       const RkCoef<float>& rk, float dt, unsigned* err, cudaStream_t);
+  cudaError_t (*background)(const MeshArg<double>&, const OpsArg<double>&, const PhysArg<double>&, const int2* faces,
+                            int n_faces, int n_walls, const double* q, double* T, double* Tv, double* grad_rho,
+                            double* G, double* Fc, double* R, unsigned* err, cudaStream_t);
+};
+ThreePassSet three_pass_p2();
+ThreePassSet three_pass_p3();
+ThreePassSet three_pass_p4();
+ThreePassSet three_pass_p5();
 
 }  // namespace chorus

@@ -18,6 +18,7 @@ struct chorus_mesh_s {
   chorus::HostMesh host;
   chorus::Tables1D tab;
   chorus::LaunchSet L{};
+  chorus::ThreePassSet L3{};
   int tile = 0;  // FP32 tile shape in use (index into the order's built tile shapes)
   chorus::OpsArg<double> ops64{};
   chorus::OpsArg<float> ops32{};
@@ -30,7 +31,10 @@ struct chorus_mesh_s {
   double* d_wJ = nullptr;  // w_i w_j w_k |J| at the solution points (reductions)
   float* d_Sf32 = nullptr;
   float* d_invJ32 = nullptr;
-  float* d_x32 = nullptr;
+  float* d_g32 = nullptr;  // x / |x|^3
+  float* d_x32 = nullptr;  // coordinates (three-pass kernels)
+  double* d_tab64 = nullptr;  // operator tables (MeshArg::tab)
+  float* d_tab32 = nullptr;
   unsigned* d_err = nullptr;
   // face list (element, local face): the interior faces from their lower element, then the wall faces
   int2* d_faces = nullptr;
@@ -41,7 +45,8 @@ struct chorus_mesh_s {
   double* d_Q0 = nullptr;     // [E][5][N3] FP64 polytrope at rest
   float* d_bg = nullptr;      // [E][2][N3]
   float* d_grho0 = nullptr;   // [E][3][N3]
-  float* d_bgT = nullptr;     // [E][6][2][N2]
+  float* d_bgT = nullptr;     // [E][6][2][N2], the other side's
+  float* d_bgTo = nullptr;    // [E][6][2][N2], the element's own (three-pass kernels)
   float* d_R0 = nullptr;      // [E][5][N3]
   double* d_red = nullptr;    // reduction partials
   // measurement: event pairs around launches while timing is enabled
@@ -102,7 +107,7 @@ struct StagePtrs {
   PhysArg<float> ph;
   BgArg bg;
   float* buf[4];  // stage buffers: u, s, A, B (ids of Stage)
-  float *Ta, *Tb, *Tv, *G, *Fc;
+  float *Ta, *Tb, *Tv, *Fc;
   const int2* faces;
   int nf, nw;
   unsigned* err;
