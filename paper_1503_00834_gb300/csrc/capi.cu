@@ -269,12 +269,25 @@ __global__ void k_reduce_partial(int64_t n_pts, int N3, const R* __restrict__ q,
     for (int c = 0; c < 6; ++c) part[blockIdx.x * 6 + c] = sh[c][0];
 }
 
-__global__ void k_reduce_final(int nb, const double* __restrict__ part, double* __restrict__ out) {
-  if (threadIdx.x < 6) {
-    double s = 0;
-    for (int b = 0; b < nb; ++b) s += part[b * 6 + threadIdx.x];
-    out[threadIdx.x] = s;
-  }
+// Blocks of the FP64 reductions' first level.
+constexpr int kRedBlocks = 1024;
+
+// Sum over the blocks' partials of component threadIdx.x < 6, in block order (the result does not depend
+// on the launch).  The whole block brings the partials into shared memory first: read from global memory
+// by the six summing threads, each batch of loads waited for the one before it.
+__device__ double sum_partials(const double* __restrict__ part) {
+  __shared__ double sh[kRedBlocks * 6];
+  for (int i = threadIdx.x; i < kRedBlocks * 6; i += blockDim.x) sh[i] = part[i];
+  __syncthreads();
+  double s = 0;
+  if (threadIdx.x < 6)
+    for (int b = 0; b < kRedBlocks; ++b) s += sh[b * 6 + threadIdx.x];
+  return s;
+}
+
+__global__ void __launch_bounds__(512) k_reduce_final(const double* __restrict__ part, double* __restrict__ out) {
+  const double s = sum_partials(part);
+  if (threadIdx.x < 6) out[threadIdx.x] = s;
 }
 
 // angular momentum L = sum w x cross m and moments of inertia I_i = sum w rho (|x|^2 - x_i^2)
@@ -311,14 +324,12 @@ __global__ void k_am_partial(int64_t n_pts, int N3, const R* __restrict__ q, con
 }
 
 // out[0..5] = (L, I) summed in a fixed order, out[6..8] = delta Omega = L / I (Eq. 33)
-__global__ void k_am_final(int nb, const double* __restrict__ part, double* __restrict__ out) {
-  if (threadIdx.x == 0) {
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int b = 0; b < nb; ++b)
-      for (int c = 0; c < 6; ++c) s[c] += part[b * 6 + c];
-    for (int c = 0; c < 6; ++c) out[c] = s[c];
-    for (int c = 0; c < 3; ++c) out[6 + c] = s[3 + c] > 0.0 ? s[c] / s[3 + c] : 0.0;
-  }
+__global__ void __launch_bounds__(512) k_am_final(const double* __restrict__ part, double* __restrict__ out) {
+  const double s = sum_partials(part);
+  if (threadIdx.x >= 32) return;
+  const double inertia = __shfl_down_sync(0xffffffffu, s, 3);
+  if (threadIdx.x < 6) out[threadIdx.x] = s;
+  if (threadIdx.x < 3) out[6 + threadIdx.x] = inertia > 0.0 ? s / inertia : 0.0;
 }
 
 // velocity update of Eq. 34 (u -= delta Omega x r), density and pressure kept
@@ -342,8 +353,6 @@ __global__ void k_am_update(int64_t n_pts, int N3, R* __restrict__ q, const doub
   for (int a = 0; a < 3; ++a) q[(e * 5 + 1 + a) * N3 + pt] = (R)mn[a];
   q[(e * 5 + 4) * N3 + pt] = (R)((double)q[(e * 5 + 4) * N3 + pt] + dke);
 }
-
-constexpr int kRedBlocks = 1024;
 
 // Arithmetic-rate probe for rooflines: every thread runs kChains independent FMA chains of `iters`
 // steps (x = x a + b) and stores their sum so that nothing is dead code.
@@ -1169,7 +1178,7 @@ chorus_status chorus_reduce(chorus_mesh m, const chorus_params* P, chorus_precis
   } else {
     return CHORUS_EINVAL;
   }
-  k_reduce_final<<<1, 32, 0, st>>>(kRedBlocks, m->d_red, m->d_red + kRedBlocks * 6);
+  k_reduce_final<<<1, 512, 0, st>>>(m->d_red, m->d_red + kRedBlocks * 6);
   CHK(cudaGetLastError());
   double r[6];
   CHK(cudaMemcpyAsync(r, m->d_red + kRedBlocks * 6, sizeof(r), cudaMemcpyDeviceToHost, st));
@@ -1192,12 +1201,12 @@ chorus_status chorus_am_correct(chorus_mesh m, const chorus_params* P, chorus_pr
   double* out = m->d_red + kRedBlocks * 6;
   if (prec == CHORUS_FP64) {
     k_am_partial<double><<<kRedBlocks, 256, 0, st>>>(nP, N3, (const double*)Q, nullptr, m->d_wJ, m->d_x64, m->d_red);
-    k_am_final<<<1, 32, 0, st>>>(kRedBlocks, m->d_red, out);
+    k_am_final<<<1, 512, 0, st>>>(m->d_red, out);
     k_am_update<double><<<grid1(nP), 256, 0, st>>>(nP, N3, (double*)Q, nullptr, m->d_x64, out + 6);
   } else if (prec == CHORUS_FP32_PERT) {
     if (!P || !m->prepared || !same_params(m->prep, *P)) return CHORUS_EINVAL;
     k_am_partial<float><<<kRedBlocks, 256, 0, st>>>(nP, N3, (const float*)Q, m->d_Q0, m->d_wJ, m->d_x64, m->d_red);
-    k_am_final<<<1, 32, 0, st>>>(kRedBlocks, m->d_red, out);
+    k_am_final<<<1, 512, 0, st>>>(m->d_red, out);
     k_am_update<float><<<grid1(nP), 256, 0, st>>>(nP, N3, (float*)Q, m->d_Q0, m->d_x64, out + 6);
   } else {
     return CHORUS_EINVAL;
@@ -1580,7 +1589,7 @@ chorus_status mesh_reduce_range(chorus_mesh_s* m, const float* Q, int64_t e0, in
   const size_t off5 = (size_t)e0 * 5 * N3, off1 = (size_t)e0 * N3;
   k_reduce_partial<float><<<kRedBlocks, 256, 0, st>>>(nP, N3, Q + off5, m->d_Q0 + off5, m->d_wJ + off1,
                                                       m->d_x64 + 3 * off1, m->d_red);
-  k_reduce_final<<<1, 32, 0, st>>>(kRedBlocks, m->d_red, m->d_red + kRedBlocks * 6);
+  k_reduce_final<<<1, 512, 0, st>>>(m->d_red, m->d_red + kRedBlocks * 6);
   CHK(cudaGetLastError());
   double r[6];
   CHK(cudaMemcpyAsync(r, m->d_red + kRedBlocks * 6, sizeof(r), cudaMemcpyDeviceToHost, st));
