@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -1074,6 +1075,43 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
   return CHORUS_OK;
 }
 
+// One device double for the loss of a chorus_closure_grad call: a word of a fixed array, marked in a mask
+// per device while the call has it (several threads and streams may be in such calls at once), or, when
+// all are taken, a stream-ordered allocation.  The call has synchronised its stream when it gives the
+// word back.  An allocation on each call cost 200 us: the default memory pool returns its memory to the
+// system at every synchronisation.
+constexpr int kLossWords = 64, kLossDevices = 64;
+__device__ double g_loss_words[kLossWords];
+std::atomic<uint64_t> g_loss_taken[kLossDevices];
+
+struct LossWord {
+  double* p = nullptr;
+  int dev = -1, word = -1;
+  cudaStream_t st;
+  explicit LossWord(cudaStream_t s) : st(s) {
+    void* base = nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    if (dev >= 0 && dev < kLossDevices && cudaGetSymbolAddress(&base, g_loss_words) == cudaSuccess) {
+      uint64_t m = g_loss_taken[dev].load();
+      while (~m != 0) {
+        const int w = __builtin_ctzll(~m);
+        if (g_loss_taken[dev].compare_exchange_weak(m, m | (uint64_t(1) << w))) {
+          word = w;
+          p = (double*)base + w;
+          return;
+        }
+      }
+    }
+    if (cudaMallocAsync((void**)&p, sizeof(double), st) != cudaSuccess) p = nullptr;
+  }
+  ~LossWord() {
+    if (word >= 0) g_loss_taken[dev].fetch_and(~(uint64_t(1) << word));
+    else if (p) cudaFreeAsync(p, st);
+  }
+  LossWord(const LossWord&) = delete;
+  LossWord& operator=(const LossWord&) = delete;
+};
+
 }  // namespace
 
 extern "C" {
@@ -1279,15 +1317,15 @@ chorus_status chorus_closure_grad(const void* weights, const float* X, const flo
                                   double* loss, void* stream) {
   if (!weights || !X || !Y || !grad || n <= 0) return CHORUS_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  double* dl = nullptr;
-  CHK(cudaMallocAsync((void**)&dl, sizeof(double), st));
-  CHK(cudaMemsetAsync(dl, 0, sizeof(double), st));
+  LossWord dl(st);
+  if (!dl.p) return CHORUS_ECUDA;
+  CHK(cudaMemsetAsync(dl.p, 0, sizeof(double), st));
   CHK(cudaMemsetAsync(grad, 0, ClosureLayout::n_params * sizeof(float), st));
-  cudaError_t e = mlp_backward(weights, X, Y, n, 0, n, grad, dl, st);
+  cudaError_t e = mlp_backward(weights, X, Y, n, 0, n, grad, dl.p, st);
   double h = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, dl, sizeof(double), cudaMemcpyDeviceToHost, st);
-  cudaFreeAsync(dl, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, dl.p, sizeof(double), cudaMemcpyDeviceToHost, st);
+  const cudaError_t se = cudaStreamSynchronize(st);  // before the word is given back
+  if (e == cudaSuccess) e = se;
   if (loss) *loss = h;
   return cu(e);
 }

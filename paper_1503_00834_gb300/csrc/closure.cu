@@ -154,10 +154,12 @@ cudaError_t launch_project(int64_t E, int Nf, int Nc, int prec, const void* Qf, 
 namespace {
 
 constexpr int NI = ClosureLayout::NI, NH = ClosureLayout::NH, NO = ClosureLayout::NO;
-constexpr int TB = 32;           // samples per CTA
-constexpr int kThreads = 256;    // 8 warps: lane = sample row, warp = column group
-constexpr int SX = NI + 2;       // odd row strides avoid bank conflicts across the 32 rows
-constexpr int SH = NH + 1;
+// Row strides of the tiles in shared memory, in words: multiples of 4 (16-byte loads along a row), the
+// rows of a weight matrix an odd number of 8-byte units apart (a warp reads 32 of them at once).
+constexpr int SX = 136;                      // inputs and outputs (135, the last column zero)
+constexpr int SH = 132;                      // hidden layers (128)
+constexpr int SW1 = 140, SW2 = 132;          // BF16: W1; W2 and W3
+constexpr int kWords = NH * SW1 > (NO + 1) * SW2 ? NH * SW1 : (NO + 1) * SW2;
 
 struct Rec {
   const __nv_bfloat16* W1;
@@ -190,62 +192,238 @@ __device__ __forceinline__ float silu_g(float z) {
   return s * (1.0f + z * (1.0f - s));
 }
 
-// out[r][c] = bias[c] + sum_k A[r][k] W[c][k] for the CTA's rows; W (bf16, [n_out][K]) staged in
-// shared memory; thread = (row, column group).
-__device__ __forceinline__ void dense(const float* A, int lda, int K, const __nv_bfloat16* Wg, const float* bias,
-                                      int n_out, __nv_bfloat16* sW, float* out, int ldo, int rows) {
-  for (int i = threadIdx.x; i < n_out * K; i += blockDim.x) sW[i] = Wg[i];
-  __syncthreads();
-  const int r = threadIdx.x % 32, grp = threadIdx.x / 32;
-  const int per = (n_out + 7) / 8;
-  const int c0 = grp * per;
-  if (r < rows) {
-    for (int c = c0; c < min(c0 + per, n_out); ++c) {
-      float acc = bias[c];
-      const __nv_bfloat16* w = sW + c * K;
-      for (int k = 0; k < K; ++k) acc += A[r * lda + k] * __bfloat162float(w[k]);
-      out[r * ldo + c] = acc;
-    }
-  }
-  __syncthreads();
-}
-
-// forward pass of TB samples; keeps the pre-activations z1, z2 and the output y in shared memory
-struct FwdSmem {
+// The tile of a CTA: TB samples, TB / 4 warps; a warp's lanes share four sample rows.
+template <int TB>
+struct Tile {
+  static constexpr int threads = 8 * TB;
   float X[TB * SX];
-  float z1[TB * SH];
+  float z1[TB * SH];  // pre-activations, then (backward) dL/dz
   float z2[TB * SH];
-  float h[TB * SH];
-  float y[TB * SX];
-  __nv_bfloat16 W[NO * NH > NH * NI ? NO * NH : NH * NI];
+  float h[TB * SH];   // the activations in use
+  float y[TB * SX];   // output, then dL/dy
+  __nv_bfloat16 W[kWords];
 };
 
-__device__ void forward_tile(const Rec& w, FwdSmem& s, int rows) {
-  dense(s.X, SX, NI, w.W1, w.b1, NH, s.W, s.z1, SH, rows);
-  for (int i = threadIdx.x; i < TB * NH; i += blockDim.x) s.h[(i / NH) * SH + i % NH] = silu_f(s.z1[(i / NH) * SH + i % NH]);
+// W1 ([NH][NI], rows of odd length) into shared memory at row stride SW1, its columns past NI zero.
+template <int TB>
+__device__ __forceinline__ void stage_w1(const __nv_bfloat16* __restrict__ Wg, __nv_bfloat16* sW) {
+  const int lane = threadIdx.x & 31;
+  const unsigned short* src = reinterpret_cast<const unsigned short*>(Wg);
+  for (int c = threadIdx.x >> 5; c < NH; c += TB / 4)
+#pragma unroll
+    for (int k = lane; k < SW1; k += 32)
+      reinterpret_cast<unsigned short*>(sW)[c * SW1 + k] = k < NI ? __ldg(src + c * NI + k) : (unsigned short)0;
+}
+
+// W2 or W3 ([ROWS][NH], a warp a row) at row stride SW2; a zero row after an odd number of rows.
+template <int TB, int ROWS>
+__device__ __forceinline__ void stage_w(const __nv_bfloat16* __restrict__ Wg, __nv_bfloat16* sW) {
+  static_assert(ClosureLayout::oW2 % 8 == 0 && ClosureLayout::oW3 % 8 == 0 && NH == 128, "rows of 32 8-byte units");
+  const int lane = threadIdx.x & 31;
+  for (int c = threadIdx.x >> 5; c < ROWS + ROWS % 2; c += TB / 4)
+    *reinterpret_cast<uint2*>(sW + c * SW2 + 4 * lane) =
+        c < ROWS ? __ldg(reinterpret_cast<const uint2*>(Wg + c * NH) + lane) : make_uint2(0u, 0u);
+}
+
+__device__ __forceinline__ void bf16x4(const __nv_bfloat16* p, float w[4]) {
+  const uint2 v = *reinterpret_cast<const uint2*>(p);
+  w[0] = __uint_as_float(v.x << 16);
+  w[1] = __uint_as_float(v.x & 0xffff0000u);
+  w[2] = __uint_as_float(v.y << 16);
+  w[3] = __uint_as_float(v.y & 0xffff0000u);
+}
+
+__device__ __forceinline__ void load4(const float* p, float v[4]) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  v[0] = t.x;
+  v[1] = t.y;
+  v[2] = t.z;
+  v[3] = t.w;
+}
+
+// out[r][c] = bias[c] + sum_k A[r][k] W[c][k], k in order, for the warp's rows: four rows by the columns
+// lane + 32 j a thread (16 sums; per four k four broadcast and four 8-byte loads for 64 products), the
+// columns past 128 one sum a lane.
+template <int K, int stride, int NCOL>
+__device__ __forceinline__ void dense(const float* A, int lda, const __nv_bfloat16* sW, const float* __restrict__ bias,
+                                      float* out, int ldo) {
+  const int lane = threadIdx.x & 31, r0 = 4 * (threadIdx.x >> 5);
+  float acc[4][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float b = __ldg(bias + lane + 32 * j);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i][j] = b;
+  }
+#pragma unroll 2
+  for (int k = 0; k < K; k += 4) {
+    float a[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) load4(A + (r0 + i) * lda + k, a[i]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float w[4];
+      bf16x4(sW + (lane + 32 * j) * stride + k, w);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) acc[i][j] = fmaf(a[i][t], w[t], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out[(r0 + i) * ldo + lane + 32 * j] = acc[i][j];
+  constexpr int X = NCOL - 128;
+  if (X > 0 && lane < 4 * X) {
+    const int r = r0 + lane / (X > 0 ? X : 1), c = 128 + lane % (X > 0 ? X : 1);
+    float s = __ldg(bias + c);
+#pragma unroll 4
+    for (int k = 0; k < K; k += 4) {
+      float a[4], w[4];
+      load4(A + r * lda + k, a);
+      bf16x4(sW + c * stride + k, w);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) s = fmaf(a[t], w[t], s);
+    }
+    out[r * ldo + c] = s;
+  }
+}
+
+// h = SiLU(z) for the warp's rows
+__device__ __forceinline__ void activate(const float* z, float* h) {
+  const int lane = threadIdx.x & 31, r0 = 4 * (threadIdx.x >> 5);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h[(r0 + i) * SH + lane + 32 * j] = silu_f(z[(r0 + i) * SH + lane + 32 * j]);
+}
+
+// Rows r0 .. of [..][135] samples into the tile (zero past `rows` and in the last column).
+template <int TB>
+__device__ __forceinline__ void load_rows(const float* __restrict__ X, int64_t r0, int rows, float* dst) {
+  for (int i = threadIdx.x; i < TB * SX; i += Tile<TB>::threads) {
+    const int r = i / SX, k = i % SX;
+    dst[i] = r < rows && k < NI ? __ldg(X + (r0 + r) * NI + k) : 0.f;
+  }
+}
+
+// Forward pass of the tile's samples: leaves z1, z2, h = SiLU(z2) and y.  A warp computes its own rows
+// of every layer; only the weights in shared memory are common.
+template <int TB>
+__device__ __forceinline__ void forward_tile(const Rec& w, Tile<TB>& s) {
+  stage_w1<TB>(w.W1, s.W);
   __syncthreads();
-  dense(s.h, SH, NH, w.W2, w.b2, NH, s.W, s.z2, SH, rows);
-  for (int i = threadIdx.x; i < TB * NH; i += blockDim.x) s.h[(i / NH) * SH + i % NH] = silu_f(s.z2[(i / NH) * SH + i % NH]);
+  dense<NI + 1, SW1, NH>(s.X, SX, s.W, w.b1, s.z1, SH);
+  __syncwarp();
+  activate(s.z1, s.h);
   __syncthreads();
-  dense(s.h, SH, NH, w.W3, w.b3, NO, s.W, s.y, SX, rows);
+  stage_w<TB, NH>(w.W2, s.W);
+  __syncthreads();
+  dense<NH, SW2, NH>(s.h, SH, s.W, w.b2, s.z2, SH);
+  __syncwarp();
+  activate(s.z2, s.h);
+  __syncthreads();
+  stage_w<TB, NO>(w.W3, s.W);
+  __syncthreads();
+  dense<NH, SW2, NO>(s.h, SH, s.W, w.b3, s.y, SX);
+}
+
+// z[r][k] <- (sum_c D[r][c] W[c][k]) SiLU'(z[r][k]), c in order to C (a multiple of four), for the warp's
+// rows (zero past `rows`): four rows by four consecutive columns a thread.
+template <int C>
+__device__ __forceinline__ void backward_data(const float* D, int ldd, const __nv_bfloat16* sW, float* z, int rows) {
+  const int lane = threadIdx.x & 31, r0 = 4 * (threadIdx.x >> 5);
+  float acc[4][4] = {};
+#pragma unroll 2
+  for (int c = 0; c < C; c += 4) {
+    float d[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) load4(D + (r0 + i) * ldd + c, d[i]);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      float w[4];
+      bf16x4(sW + (c + t) * SW2 + 4 * lane, w);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[i][u] = fmaf(d[i][t], w[u], acc[i][u]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float v[4];
+    load4(z + (r0 + i) * SH + 4 * lane, v);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = r0 + i < rows ? acc[i][u] * silu_g(v[u]) : 0.f;
+    *reinterpret_cast<float4*>(z + (r0 + i) * SH + 4 * lane) = make_float4(v[0], v[1], v[2], v[3]);
+  }
+}
+
+// gW[c][k] += sum_r D[r][c] A[r][k] over the tile, c < NC, k < NK: up to 128 x 128 eight c by four
+// consecutive k a thread (32 sums; per sample two broadcast and one 16-byte load), the rows and columns
+// past that one sum a thread; gb[c] += sum_r D[r][c].  v4: the rows of gW are 16-byte aligned (vector
+// atomics).
+template <int TB, int NC, int NK>
+__device__ __forceinline__ void backward_weights(const float* D, int ldd, const float* A, int lda, float* gW, float* gb,
+                                                 bool v4) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int c0 = 8 * warp; c0 < 128; c0 += 2 * TB) {
+    float acc[8][4] = {};
+#pragma unroll 4
+    for (int r = 0; r < TB; ++r) {
+      float d[8], a[4];
+      load4(D + r * ldd + c0, d);
+      load4(D + r * ldd + c0 + 4, d + 4);
+      load4(A + r * lda + 4 * lane, a);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[i][u] = fmaf(d[i], a[u], acc[i][u]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float* g = gW + (size_t)(c0 + i) * NK + 4 * lane;
+      if (v4) {
+        atomicAdd(reinterpret_cast<float4*>(g), make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) atomicAdd(g + u, acc[i][u]);
+      }
+    }
+  }
+  constexpr int XC = NC - 128, XK = NK - 128;
+  static_assert(XC == 0 || XK == 0, "one of the two is 128");
+  for (int i = threadIdx.x; i < XC * 128 + XK * 128; i += Tile<TB>::threads) {
+    const int c = XC > 0 ? 128 + i / 128 : i / (XK > 0 ? XK : 1), k = XC > 0 ? i % 128 : 128 + i % (XK > 0 ? XK : 1);
+    float s = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < TB; ++r) s = fmaf(D[r * ldd + c], A[r * lda + k], s);
+    atomicAdd(gW + (size_t)c * NK + k, s);
+  }
+  for (int c = threadIdx.x; c < NC; c += Tile<TB>::threads) {
+    float s = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < TB; ++r) s += D[r * ldd + c];
+    atomicAdd(gb + c, s);
+  }
 }
 
 }  // namespace
 
 // Y = MLP(X) for n samples ([n][135] FP32, row-major).
-__global__ void k_mlp_forward(const void* weights, const float* __restrict__ X, float* __restrict__ Y, int64_t n) {
+template <int TB>
+__global__ void __launch_bounds__(Tile<TB>::threads)
+    k_mlp_forward(const void* weights, const float* __restrict__ X, float* __restrict__ Y, int64_t n) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  FwdSmem& s = *reinterpret_cast<FwdSmem*>(smraw);
+  Tile<TB>& s = *reinterpret_cast<Tile<TB>*>(smraw);
   const Rec w = rec_of(weights);
   const int64_t r0 = (int64_t)blockIdx.x * TB;
   const int rows = (int)((n - r0) < TB ? (n - r0) : TB);
-  for (int i = threadIdx.x; i < TB * NI; i += blockDim.x) {
-    const int r = i / NI, k = i % NI;
-    s.X[r * SX + k] = r < rows ? X[(r0 + r) * NI + k] : 0.f;
-  }
+  load_rows<TB>(X, r0, rows, s.X);
+  forward_tile<TB>(w, s);
   __syncthreads();
-  forward_tile(w, s, rows);
-  for (int i = threadIdx.x; i < rows * NO; i += blockDim.x) Y[(r0 + i / NO) * NO + i % NO] = s.y[(i / NO) * SX + i % NO];
+  for (int i = threadIdx.x; i < rows * NO; i += Tile<TB>::threads) Y[r0 * NO + i] = s.y[(i / NO) * SX + i % NO];
 }
 
 // Training pairs: X = q'_c / in_scale, Y = (P R_f - R_c) / out_scale per element.
@@ -264,103 +442,54 @@ __global__ void k_make_pairs(const void* weights, const R* __restrict__ Qc, cons
 }
 
 // Gradient of L = sum (y - t)^2 / (2 n_total) over the CTA's samples, accumulated into
-// grad (FP32, layout of ClosureLayout::master) with atomics; loss partial into *loss.
-__global__ void k_mlp_backward(const void* weights, const float* __restrict__ X, const float* __restrict__ T,
-                               int64_t n, int64_t row0, int64_t rows_total, float* __restrict__ grad,
-                               double* __restrict__ loss) {
+// grad (FP32, layout of ClosureLayout::master) with atomics; loss partial into *loss.  FP32 products
+// (bound by the FMA rate: 2.5 GFLOP for 8,192 samples, 32 us at 78 TFLOP/s): register tiles of 16 and 32
+// sums a thread, everything between the global inputs and the atomics in shared memory.
+template <int TB>
+__global__ void __launch_bounds__(Tile<TB>::threads)
+    k_mlp_backward(const void* weights, const float* __restrict__ X, const float* __restrict__ T, int64_t row0,
+                   int64_t rows_total, float* __restrict__ grad, double* __restrict__ loss) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  FwdSmem& s = *reinterpret_cast<FwdSmem*>(smraw);
-  float* h1 = reinterpret_cast<float*>(smraw + sizeof(FwdSmem));  // [TB][SH]
+  Tile<TB>& s = *reinterpret_cast<Tile<TB>*>(smraw);
   const Rec w = rec_of(weights);
   const int64_t r0 = row0 + (int64_t)blockIdx.x * TB;
   const int64_t left = row0 + rows_total - r0;
   const int rows = (int)(left < 0 ? 0 : (left < TB ? left : TB));
-  for (int i = threadIdx.x; i < TB * NI; i += blockDim.x) {
-    const int r = i / NI, k = i % NI;
-    s.X[r * SX + k] = r < rows ? X[(r0 + r) * NI + k] : 0.f;
-  }
+  load_rows<TB>(X, r0, rows, s.X);
+  forward_tile<TB>(w, s);
   __syncthreads();
-  forward_tile(w, s, rows);
-  // h1 = silu(z1), h2 = silu(z2) (s.h holds h2 after the forward pass)
-  for (int i = threadIdx.x; i < TB * NH; i += blockDim.x) h1[(i / NH) * SH + i % NH] = silu_f(s.z1[(i / NH) * SH + i % NH]);
-  // dY = (y - t) / n_total, loss partial
+  // dY = (y - t) / n_total, loss partial (y's last column becomes zero)
   const double inv_n = 1.0 / ((double)rows_total * NO);
   double lp = 0.0;
-  for (int i = threadIdx.x; i < TB * NO; i += blockDim.x) {
-    const int r = i / NO, k = i % NO;
+  for (int i = threadIdx.x; i < TB * SX; i += Tile<TB>::threads) {
+    const int r = i / SX, k = i % SX;
     float d = 0.f;
-    if (r < rows) {
-      const float diff = s.y[r * SX + k] - T[(r0 + r) * NO + k];
+    if (r < rows && k < NO) {
+      const float diff = s.y[i] - __ldg(T + (r0 + r) * NO + k);
       lp += 0.5 * (double)diff * diff;
       d = (float)(diff * inv_n);
     }
-    s.y[r * SX + k] = d;  // y now holds dY
+    s.y[i] = d;  // y now holds dY
   }
-  atomicAdd(loss, lp * inv_n);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) lp += __shfl_xor_sync(0xffffffffu, lp, o);
+  if ((threadIdx.x & 31) == 0) atomicAdd(loss, lp * inv_n);
   __syncthreads();
-  float* gW1 = grad + ClosureLayout::mW1;
-  float* gW2 = grad + ClosureLayout::mW2;
-  float* gW3 = grad + ClosureLayout::mW3;
-  float* gb1 = grad + ClosureLayout::mb1;
-  float* gb2 = grad + ClosureLayout::mb2;
-  float* gb3 = grad + ClosureLayout::mb3;
-  // dW3[c][k] = sum_r dY[r][c] h2[r][k];  db3[c] = sum_r dY[r][c]
-  for (int i = threadIdx.x; i < NO * NH; i += blockDim.x) {
-    const int c = i / NH, k = i % NH;
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc += s.y[r * SX + c] * s.h[r * SH + k];
-    atomicAdd(gW3 + i, acc);
-  }
-  for (int c = threadIdx.x; c < NO; c += blockDim.x) {
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc += s.y[r * SX + c];
-    atomicAdd(gb3 + c, acc);
-  }
-  // dz2[r][k] = (sum_c dY[r][c] W3[c][k]) silu'(z2[r][k])  -> stored in z2
-  for (int i = threadIdx.x; i < NO * NH; i += blockDim.x) s.W[i] = w.W3[i];
+  const bool v4 = ((uintptr_t)grad & 15u) == 0;
+  static_assert(ClosureLayout::mW2 % 4 == 0 && ClosureLayout::mW3 % 4 == 0, "aligned rows of W2, W3");
+  // dW3 = dY^T h2, db3; dz2 = (dY W3) SiLU'(z2) in place (W3 is still staged)
+  backward_weights<TB, NO, NH>(s.y, SX, s.h, SH, grad + ClosureLayout::mW3, grad + ClosureLayout::mb3, v4);
+  backward_data<NO + 1>(s.y, SX, s.W, s.z2, rows);
   __syncthreads();
-  for (int i = threadIdx.x; i < TB * NH; i += blockDim.x) {
-    const int r = i / NH, k = i % NH;
-    float acc = 0.f;
-    for (int c = 0; c < NO; ++c) acc += s.y[r * SX + c] * __bfloat162float(s.W[c * NH + k]);
-    s.z2[r * SH + k] = r < rows ? acc * silu_g(s.z2[r * SH + k]) : 0.f;
-  }
+  // dW2 = dz2^T h1, db2; dz1 = (dz2 W2) SiLU'(z1) in place
+  activate(s.z1, s.h);
+  stage_w<TB, NH>(w.W2, s.W);
   __syncthreads();
-  // dW2[c][k] = sum_r dz2[r][c] h1[r][k]
-  for (int i = threadIdx.x; i < NH * NH; i += blockDim.x) {
-    const int c = i / NH, k = i % NH;
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc += s.z2[r * SH + c] * h1[r * SH + k];
-    atomicAdd(gW2 + i, acc);
-  }
-  for (int c = threadIdx.x; c < NH; c += blockDim.x) {
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc += s.z2[r * SH + c];
-    atomicAdd(gb2 + c, acc);
-  }
-  // dz1[r][k] = (sum_c dz2[r][c] W2[c][k]) silu'(z1[r][k])  -> stored in z1
+  backward_weights<TB, NH, NH>(s.z2, SH, s.h, SH, grad + ClosureLayout::mW2, grad + ClosureLayout::mb2, v4);
+  backward_data<NH>(s.z2, SH, s.W, s.z1, rows);
   __syncthreads();
-  for (int i = threadIdx.x; i < NH * NH; i += blockDim.x) s.W[i] = w.W2[i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < TB * NH; i += blockDim.x) {
-    const int r = i / NH, k = i % NH;
-    float acc = 0.f;
-    for (int c = 0; c < NH; ++c) acc += s.z2[r * SH + c] * __bfloat162float(s.W[c * NH + k]);
-    h1[r * SH + k] = r < rows ? acc * silu_g(s.z1[r * SH + k]) : 0.f;  // h1 now holds dz1
-  }
-  __syncthreads();
-  // dW1[c][k] = sum_r dz1[r][c] X[r][k]
-  for (int i = threadIdx.x; i < NH * NI; i += blockDim.x) {
-    const int c = i / NI, k = i % NI;
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc += h1[r * SH + c] * s.X[r * SX + k];
-    atomicAdd(gW1 + i, acc);
-  }
-  for (int c = threadIdx.x; c < NH; c += blockDim.x) {
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc += h1[r * SH + c];
-    atomicAdd(gb1 + c, acc);
-  }
+  // dW1 = dz1^T X, db1 (rows of 135: scalar atomics)
+  backward_weights<TB, NH, NI>(s.z1, SH, s.X, SX, grad + ClosureLayout::mW1, grad + ClosureLayout::mb1, false);
 }
 
 // Adam update of the FP32 master parameters; writes the BF16 weights and FP32 biases of the record.
@@ -386,30 +515,49 @@ __global__ void k_load_master(const void* weights, float* __restrict__ master) {
   master[i] = closure_load_param(weights, i);
 }
 
-size_t mlp_smem_bytes(bool backward) {
-  return sizeof(FwdSmem) + (backward ? sizeof(float) * TB * SH : 0);
-}
-
 template __global__ void k_make_pairs<float>(const void*, const float*, const double*, const float*, const float*,
                                              float*, float*, int64_t);
 template __global__ void k_make_pairs<double>(const void*, const double*, const double*, const double*,
                                               const double*, float*, float*, int64_t);
 
-cudaError_t mlp_forward(const void* weights, const float* X, float* Y, int64_t n, cudaStream_t st) {
-  const size_t sm = mlp_smem_bytes(false);
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+namespace {
+
+template <int TB>
+cudaError_t forward_tb(const void* weights, const float* X, float* Y, int64_t n, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_forward<TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Tile<TB>));
   if (e != cudaSuccess) return e;
-  k_mlp_forward<<<(unsigned)((n + TB - 1) / TB), kThreads, sm, st>>>(weights, X, Y, n);
+  k_mlp_forward<TB><<<(unsigned)((n + TB - 1) / TB), Tile<TB>::threads, sizeof(Tile<TB>), st>>>(weights, X, Y, n);
   return cudaGetLastError();
+}
+
+template <int TB>
+cudaError_t backward_tb(const void* weights, const float* X, const float* T, int64_t row0, int64_t rows, float* grad,
+                        double* loss, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_backward<TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Tile<TB>));
+  if (e != cudaSuccess) return e;
+  k_mlp_backward<TB><<<(unsigned)((rows + TB - 1) / TB), Tile<TB>::threads, sizeof(Tile<TB>), st>>>(weights, X, T, row0,
+                                                                                                  rows, grad, loss);
+  return cudaGetLastError();
+}
+
+// Samples per CTA: one CTA per SM either way (its shared memory), so the largest tile, which stages the
+// weights and adds the gradients the fewest times, once its CTAs fill half the chip; below that smaller
+// tiles, so that a batch of a thousand still spreads over the SMs.
+constexpr int64_t kWide = 64 * 76, kMid = 32 * 76;
+
+}  // namespace
+
+cudaError_t mlp_forward(const void* weights, const float* X, float* Y, int64_t n, cudaStream_t st) {
+  return n >= kWide  ? forward_tb<64>(weights, X, Y, n, st)
+         : n >= kMid ? forward_tb<32>(weights, X, Y, n, st)
+                     : forward_tb<16>(weights, X, Y, n, st);
 }
 
 cudaError_t mlp_backward(const void* weights, const float* X, const float* T, int64_t n, int64_t row0, int64_t rows,
                          float* grad, double* loss, cudaStream_t st) {
-  const size_t sm = mlp_smem_bytes(true);
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  k_mlp_backward<<<(unsigned)((rows + TB - 1) / TB), kThreads, sm, st>>>(weights, X, T, n, row0, rows, grad, loss);
-  return cudaGetLastError();
+  return rows >= kWide  ? backward_tb<64>(weights, X, T, row0, rows, grad, loss, st)
+         : rows >= kMid ? backward_tb<32>(weights, X, T, row0, rows, grad, loss, st)
+                        : backward_tb<16>(weights, X, T, row0, rows, grad, loss, st);
 }
 
 cudaError_t make_pairs(int prec, const void* weights, const void* Qc, const double* Q0, const void* PRf,
