@@ -7,10 +7,13 @@
 // applied in FP32 to the accumulator.  Element inputs are scaled by the reciprocal of the input
 // scale (FP32; FP64 where the background is subtracted first).
 //
-// Work decomposition: persistent CTAs of 128 threads; a tile is 128 samples (the MMA M).  The three
+// Work decomposition: persistent CTAs of 512 threads; a tile is 128 samples (the MMA M).  The three
 // weight matrices are copied once per CTA into shared memory in the MMA operand layout; per tile
 // the inputs are converted into the A operand, and the three products run back to back, each
-// followed by an epilogue in which warp w reads TMEM lanes 32w..32w+31 (its tile rows).
+// followed by an epilogue in which warp w reads TMEM lanes 32 (w % 4) .. + 31 (its tile rows) and its
+// share w / 4 of the columns.  The products are 1 % of a tile's time: conversions, SiLU and stores bound
+// it, one tile's chain after another, so the chain is spread over sixteen warps and the next tile's
+// inputs are loaded while it runs (FP32; 8,192 samples: 25 us, 111 us with four warps).
 //
 // Operand layout (K-major, no swizzle): 8 x 8 BF16 core matrices of 128 contiguous bytes (8 rows of
 // 16 bytes); the core matrix of row group g and K chunk c of an R x K operand starts at byte
@@ -30,6 +33,9 @@ constexpr int NI = ClosureLayout::NI, NH = ClosureLayout::NH, NO = ClosureLayout
 constexpr int KA = 144;   // 135 inputs padded to a multiple of 16 (the MMA K step)
 constexpr int NOP = 144;  // 135 outputs padded to a multiple of 16 (MMA N)
 constexpr int kTmemCols = 256;
+constexpr int kThreads = 512;
+constexpr int kChunks = TM * (KA / 8);                            // 8-input chunks of a tile
+constexpr int kPer = (kChunks + kThreads - 1) / kThreads;         // of a thread
 
 // shared-memory plan (bytes); every operand block starts on a 1024-byte boundary
 constexpr int oW1 = 0;                       // [NH][KA]
@@ -38,7 +44,7 @@ constexpr int oW3 = oW2 + NH * NH * 2;       // [NOP][NH]
 constexpr int oA = oW3 + NOP * NH * 2;       // [TM][KA]   layer-1 input
 constexpr int oH = oA + TM * KA * 2;         // [TM][NH]   layer-2 / layer-3 input
 constexpr int oEnd = oH + TM * NH * 2;
-constexpr int kOutStride = NO;               // FP32 output staging rows (overlays A and H); odd stride
+constexpr int kOutStride = NO;               // FP32 output staging rows (overlays A and H), as in global memory; odd stride
 static_assert(TM * kOutStride * 4 <= oEnd - oA, "output staging must fit in the A and H blocks");
 static_assert(oW2 % 1024 == 0 && oW3 % 1024 == 0 && oA % 1024 == 0 && oH % 1024 == 0, "operand alignment");
 constexpr size_t kSmemBytes = (size_t)oEnd + 1024;  // + alignment slack
@@ -140,22 +146,32 @@ __device__ __forceinline__ Rec rec_of(const void* w) {
   return r;
 }
 
-// copy a row-major [n_out][n_in] BF16 matrix into the operand block [n_pad][k_pad], zero-padded
-__device__ void stage_weights(const __nv_bfloat16* W, int n_out, int n_in, int n_pad, int k_pad, __nv_bfloat16* dst) {
-  for (int i = threadIdx.x; i < n_pad * k_pad; i += blockDim.x) {
-    const int n = i / k_pad, k = i % k_pad;
-    dst[opnd(n, k, k_pad)] = (n < n_out && k < n_in) ? W[n * n_in + k] : __float2bfloat16_rn(0.0f);
+// copy a row-major [n_out][n_in] BF16 matrix into the operand block [n_pad][k_pad], zero-padded, one
+// 16-byte core-matrix row at a time (vec: the source's rows are whole, aligned 16-byte units)
+__device__ void stage_weights(const __nv_bfloat16* W, int n_out, int n_in, int n_pad, int k_pad, bool vec,
+                              __nv_bfloat16* dst) {
+  for (int i = threadIdx.x; i < n_pad * (k_pad / 8); i += kThreads) {
+    const int n = i / (k_pad / 8), k = 8 * (i % (k_pad / 8));
+    __align__(16) __nv_bfloat16 v[8];
+    if (vec && n < n_out && k + 8 <= n_in) {
+      *reinterpret_cast<uint4*>(v) = __ldg(reinterpret_cast<const uint4*>(W + n * n_in + k));
+    } else {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = (n < n_out && k + u < n_in) ? W[n * n_in + k + u] : __float2bfloat16_rn(0.0f);
+    }
+    *reinterpret_cast<uint4*>(dst + opnd(n, k, k_pad)) = *reinterpret_cast<const uint4*>(v);
   }
 }
 
-// Epilogue of a hidden layer: z = acc + b, h = SiLU(z), written as BF16 into the H operand block.
-__device__ __forceinline__ void hidden_epilogue(uint32_t tmem, int col0, const float* bias, __nv_bfloat16* H) {
-  const int w = threadIdx.x >> 5, row = threadIdx.x;
-  const uint32_t lane = (uint32_t)(32 * w) << 16;
+// Epilogue of a hidden layer: z = acc + b, h = SiLU(z), written as BF16 into the H operand block.  The
+// warp's 32 rows and 32 columns.
+__device__ __forceinline__ void hidden_epilogue(uint32_t tmem, const float* bias, __nv_bfloat16* H) {
+  const int w = threadIdx.x >> 5, q = w & 3, row = 32 * q + (threadIdx.x & 31);
+  const uint32_t lane = (uint32_t)(32 * q) << 16;
 #pragma unroll 1
-  for (int c = 0; c < NH; c += 16) {
+  for (int c = 32 * (w >> 2); c < 32 * (w >> 2) + 32; c += 16) {
     float v[16];
-    tmem_ld16(tmem + lane + (uint32_t)(col0 + c), v);
+    tmem_ld16(tmem + lane + (uint32_t)c, v);
     __align__(16) __nv_bfloat16 h[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) h[i] = __float2bfloat16_rn(silu(v[i] + __ldg(bias + c + i)));
@@ -170,7 +186,7 @@ __device__ __forceinline__ void hidden_epilogue(uint32_t tmem, int col0, const f
 // in_scale per variable; false reads sample rows X[r][135] as they are.  Output: ELEM = true writes
 // or adds out_scale * y into R[e][135]; false stores y into Y[r][135].
 template <bool ELEM, class R>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kThreads, 1)
     k_mlp_tc(const void* weights, const R* __restrict__ Q, const double* __restrict__ Q0, R* __restrict__ out,
              int64_t n, int accumulate, unsigned* err) {
   extern __shared__ unsigned char smraw[];
@@ -198,9 +214,10 @@ __global__ void __launch_bounds__(128, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  stage_weights(w.W[0], NH, NI, NH, KA, sW1);
-  stage_weights(w.W[1], NH, NH, NH, NH, sW2);
-  stage_weights(w.W[2], NO, NH, NOP, NH, sW3);
+  const bool vec = ((uintptr_t)w.W[1] & 15u) == 0 && ((uintptr_t)w.W[2] & 15u) == 0;
+  stage_weights(w.W[0], NH, NI, NH, KA, false, sW1);  // rows of 270 bytes
+  stage_weights(w.W[1], NH, NH, NH, NH, vec, sW2);
+  stage_weights(w.W[2], NO, NH, NOP, NH, vec, sW3);
   fence_before();
   __syncthreads();
   fence_after();
@@ -208,39 +225,67 @@ __global__ void __launch_bounds__(128, 1)
   const uint32_t dA = tmem, dB = tmem + 128;  // accumulator columns: layers 1 and 3 in [0, 144), layer 2 in [128, 256)
   uint32_t phase = 0;
   const int64_t n_tiles = (n + TM - 1) / TM;
-  float inv_in[5];
-  double inv_in64[5];
+  // per-variable scales (indexed at run time: in shared memory)
+  __shared__ float inv_in[5], out_sc[5];
+  __shared__ double inv_in64[5];
+  if (threadIdx.x < 5) {
+    inv_in64[threadIdx.x] = 1.0 / (double)__ldg(w.in_scale + threadIdx.x);
+    inv_in[threadIdx.x] = (float)inv_in64[threadIdx.x];
+    out_sc[threadIdx.x] = __ldg(w.out_scale + threadIdx.x);
+  }
+  __syncthreads();
+
+  // A thread's 8-input chunks of a tile: chunk i is row i / 18, inputs 8 (i % 18) .. + 7 (consecutive
+  // threads read consecutive 32-byte pieces).
+  auto load = [&](const auto* src, int64_t tile, int j, auto(&x)[8]) {
+    const int64_t r0 = tile * TM;
+    const int rows = (int)((n - r0) < TM ? (n - r0) : TM);
+    const int i = threadIdx.x + j * kThreads, r = i / (KA / 8), c = i % (KA / 8);
 #pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    inv_in64[v] = 1.0 / (double)__ldg(w.in_scale + v);
-    inv_in[v] = (float)inv_in64[v];
+    for (int u = 0; u < 8; ++u)
+      x[u] = i < kChunks && r < rows && 8 * c + u < NI ? src[(r0 + r) * NI + 8 * c + u] : 0;
+  };
+  constexpr bool AHEAD = sizeof(R) == 4;  // FP32: the next tile's inputs are loaded during this tile
+  R x[AHEAD ? kPer : 1][8];
+  if constexpr (AHEAD) {
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) load(Q, blockIdx.x, j, x[j]);
   }
 
   for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
     const int64_t r0 = t * TM;
     const int rows = (int)((n - r0) < TM ? (n - r0) : TM);
-    // ---- layer-1 input, one 8-column chunk per thread step: 8 consecutive inputs of a row (coalesced
-    // across the warp), scaled, rounded to BF16, stored as one 16-byte row of a core matrix
-#pragma unroll 6
-    for (int i = threadIdx.x; i < TM * (KA / 8); i += blockDim.x) {  // 18 steps: six chunks' loads in flight
+    // ---- layer-1 input: scaled, rounded to BF16, stored as 16-byte rows of the core matrices
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const int i = threadIdx.x + j * kThreads;
+      if (i >= kChunks) break;
+      R(&xj)[8] = x[AHEAD ? j : 0];
+      double x0[8];
+      if constexpr (!AHEAD) {
+        load(Q, t, j, xj);
+        if (Q0) load(Q0, t, j, x0);
+      }
       const int r = i / (KA / 8), c = i % (KA / 8);
       __align__(16) __nv_bfloat16 v[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int k = 8 * c + u;
-        float x = 0.0f;
-        if (r < rows && k < NI) {
-          const int64_t gi = (r0 + r) * NI + k;
-          if (ELEM) {
-            if (Q0) x = (float)(((double)Q[gi] - Q0[gi]) * inv_in64[k / 27]);  // the difference needs FP64
-            else x = (float)Q[gi] * inv_in[k / 27];
-          } else {
-            x = (float)Q[gi];
-          }
+        float f = (float)xj[u];
+        if (ELEM) {
+          const int var = k / 27 < 5 ? k / 27 : 4;
+          if (!AHEAD && Q0) f = (float)(((double)xj[u] - x0[u]) * inv_in64[var]);  // the difference needs FP64
+          else f *= inv_in[var];
         }
-        v[u] = __float2bfloat16_rn(x);
+        v[u] = __float2bfloat16_rn(f);
       }
       *reinterpret_cast<uint4*>(sA + opnd(r, 8 * c, KA)) = *reinterpret_cast<const uint4*>(v);
+    }
+    if constexpr (AHEAD) {
+      if (t + gridDim.x < n_tiles) {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) load(Q, t + gridDim.x, j, x[j]);
+      }
     }
     fence_async_smem();
     fence_before();
@@ -266,34 +311,35 @@ __global__ void __launch_bounds__(128, 1)
       if (abort_flag) break;
       fence_after();
       if (layer < 2) {
-        hidden_epilogue(layer == 1 ? dB : dA, 0, w.b[layer], sH);
+        hidden_epilogue(layer == 1 ? dB : dA, w.b[layer], sH);
         fence_async_smem();
         fence_before();
         __syncthreads();
       } else {
-        // output layer: y = acc + b3 (columns 0..134), staged as FP32 rows for coalesced stores
-        const int row = threadIdx.x;
-        const uint32_t lane = (uint32_t)(32 * warp) << 16;
+        // output layer: y = acc + b3 (columns 0..134), times the output scale for elements, staged as FP32
+        // rows for coalesced stores: the staged tile is the output's rows r0 .. as they lie in memory
+        const int q = warp & 3, row = 32 * q + (threadIdx.x & 31);
+        const uint32_t lane = (uint32_t)(32 * q) << 16;
 #pragma unroll 1
-        for (int c = 0; c < NOP; c += 16) {
+        for (int c = 16 * (warp >> 2); c < NOP; c += 64) {
           float v[16];
           tmem_ld16(dA + lane + (uint32_t)c, v);
 #pragma unroll
           for (int i = 0; i < 16; ++i)
-            if (c + i < NO) sOut[row * kOutStride + c + i] = v[i] + __ldg(w.b[2] + c + i);
+            if (c + i < NO) {
+              const float y = v[i] + __ldg(w.b[2] + c + i);
+              sOut[row * kOutStride + c + i] = ELEM ? y * out_sc[(c + i) / 27] : y;
+            }
         }
         fence_before();
         __syncthreads();
-        for (int i = threadIdx.x; i < rows * NO; i += blockDim.x) {
-          const int r = i / NO, k = i % NO;
-          const float y = sOut[r * kOutStride + k];
-          R* o = out + (r0 + r) * NO + k;
-          if (ELEM) {
-            const R c = (R)(y * __ldg(w.out_scale + k / 27));
-            *o = accumulate ? *o + c : c;
-          } else {
-            *o = (R)y;
-          }
+        R* o = out + r0 * NO;
+        if (ELEM && accumulate) {
+#pragma unroll 4
+          for (int i = threadIdx.x; i < rows * NO; i += kThreads) o[i] += (R)sOut[i];
+        } else {
+#pragma unroll 4
+          for (int i = threadIdx.x; i < rows * NO; i += kThreads) o[i] = (R)sOut[i];
         }
         __syncthreads();  // the staging rows overlay the next tile's A block
       }
@@ -324,7 +370,7 @@ cudaError_t launch_tc(const void* weights, const R* Q, const double* Q0, R* out,
   if (e != cudaSuccess) return e;
   const int64_t tiles = (n + TM - 1) / TM;
   const unsigned grid = (unsigned)(tiles < sm_count() ? tiles : sm_count());
-  k_mlp_tc<ELEM, R><<<grid, 128, kSmemBytes, st>>>(weights, Q, Q0, out, n, accumulate, err);
+  k_mlp_tc<ELEM, R><<<grid, kThreads, kSmemBytes, st>>>(weights, Q, Q0, out, n, accumulate, err);
   return cudaGetLastError();
 }
 
