@@ -41,6 +41,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
 }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// Programmatic dependent launch: let the next kernel of the stream start; wait until the kernel before it
+// has completed (both do nothing in a launch without the attribute).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Polls of a bounded mbarrier wait when the mesh sets no limit of its own (about a second with the
 // back-off below).
 constexpr uint32_t kDefaultWaitPolls = 1u << 24;

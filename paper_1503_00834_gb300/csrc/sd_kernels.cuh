@@ -26,6 +26,7 @@
 // the computed arrays are XOR-swizzled so that xi-, eta- and zeta-line accesses are conflict free.
 #pragma once
 #include <type_traits>
+#include <utility>
 
 #include "sd_device.cuh"
 #include "sd_physics.cuh"
@@ -103,7 +104,9 @@ struct Layout {
   static constexpr int block(int n) { return padded ? EPB * stride(n) : (EPB * n + 2 * V + V - 1) / V * V; }
   static constexpr bool SM = stage_metrics<N, R>();
   static constexpr int SQ = stride(5 * N3), SBG = stride(2 * N3), SGR0 = stride(3 * N3);
-  static constexpr int SG = padded ? pad_stride<R>(16 * N3) : 16 * N3;
+  // N = 3 FP32: 443 words, 27 mod 32, so that the xi lines of a warp's elements start in 32 different
+  // banks (0.206 -> 0.193 ms at 98,304 elements); no stride measured better at N = 5 and 6
+  static constexpr int SG = padded ? pad_stride<R>(16 * N3) : 16 * N3 + (N == 3 && sizeof(R) == 4 ? 11 : 0);
   // interpolation I[f][s] and derivative D[i][f] as pairs of equal values, indexed by rolled loops
   static constexpr int TAB = 4 * (N + 1) * N;
   static constexpr int oI = 0;
@@ -350,7 +353,6 @@ __device__ __forceinline__ bool stage_elements(const KArgs<R>& A, R* sm, uint64_
     if (L::SM) bytes += si.bytes(ne) + 2 * ne * L::SS * sizeof(R);
     if (tid == 0 && bytes > 0) {
       mbar_expect_tx(bar, bytes);
-      sq.issue(dq, A.q, e0, ne, L::SQ, bar);
       if constexpr (L::SM) {
         issue_metrics<N, R, L>(A.m.Sf, e0, ne, 2, sm + L::oS0 + u0 * L::SS, bar);
         si.issue(di, A.m.invJ, e0, ne, L::SIJ, bar);
@@ -364,8 +366,9 @@ __device__ __forceinline__ bool stage_elements(const KArgs<R>& A, R* sm, uint64_
     if (L::SM) si.rest(di, A.m.invJ, e0, ne, L::SIJ, tid, nt);
   } else if (tid == 0 && bytes > 0) {
     mbar_expect_tx(bar, bytes);
-    sq.issue(dq, A.q, e0, ne, L::SQ, bar);
   }
+  pdl_wait();  // the mesh's own data above; the state and its traces come from the kernels before
+  if (tid == 0) sq.issue(dq, A.q, e0, ne, L::SQ, bar);
   sq.rest(dq, A.q, e0, ne, L::SQ, tid, nt);
   between();
   bool ok = true;
@@ -1043,6 +1046,7 @@ template <int N, bool PERT, class R, int EPB, int MODE, bool KR>
 __global__ void __launch_bounds__(EPB * N * N, sizeof(R) == 4 ? vol_min_blocks<N, EPB>() : 1) k_vol(const KArgs<R> A) {
   constexpr int units = (EPB + unit_elems<N, EPB>() - 1) / unit_elems<N, EPB>();
   __shared__ __align__(8) uint64_t bars[units * kVolBars];
+  pdl_trigger();
   if (threadIdx.x < units * kVolBars) mbar_init(&bars[threadIdx.x]);
   __syncthreads();
   uint32_t ph = 0;
@@ -1078,17 +1082,20 @@ __device__ __forceinline__ void face_point(const KArgs<R>& A, const int2* __rest
   const size_t oR = wall ? oL : (size_t)k * 6 + Fn;
   R qL[5], tvL[4], So[3], qR[5], tvR[4];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) qR[v] = __ldg(A.T + (oL * 5 + v) * N2 + t);
-#pragma unroll
-  for (int v = 0; v < 4; ++v) tvL[v] = __ldg(A.Tv + (oL * 4 + v) * N2 + t);
+  for (int n = 0; n < 3; ++n)
+    So[n] = sgn * __ldg(A.m.Sf + (((size_t)e * 3 + D) * 3 * (N + 1) + n * (N + 1) + (side ? N : 0)) * N2 + t);
   R r0L = R(0), E0L = R(0), r0R = R(0), E0R = R(0);
   if (PERT) {
     r0R = (R)__ldg(A.bg.bgT + (oL * 2) * N2 + t);
     E0R = (R)__ldg(A.bg.bgT + (oL * 2 + 1) * N2 + t);
+    r0L = (R)__ldg(A.bg.bgT + (oR * 2) * N2 + tp);
+    E0L = (R)__ldg(A.bg.bgT + (oR * 2 + 1) * N2 + tp);
   }
-  const R* Sl = A.m.Sf + ((size_t)e * 3 + D) * 3 * (N + 1) * N2;
+  pdl_wait();
 #pragma unroll
-  for (int n = 0; n < 3; ++n) So[n] = sgn * __ldg(Sl + (n * (N + 1) + (side ? N : 0)) * N2 + t);
+  for (int v = 0; v < 5; ++v) qR[v] = __ldg(A.T + (oL * 5 + v) * N2 + t);
+#pragma unroll
+  for (int v = 0; v < 4; ++v) tvL[v] = __ldg(A.Tv + (oL * 4 + v) * N2 + t);
   if (wall) {  // exact inviscid flux (0, p S, 0) minus the normal viscous traction; energy: f.S
     const Pt<R> st = point_state<PERT>(qR, r0R, E0R, A.ph);
     const R mag2 = dot3(So, So);
@@ -1103,10 +1110,6 @@ __device__ __forceinline__ void face_point(const KArgs<R>& A, const int2* __rest
   for (int v = 0; v < 5; ++v) qL[v] = __ldg(A.T + (oR * 5 + v) * N2 + tp);
 #pragma unroll
   for (int v = 0; v < 4; ++v) tvR[v] = __ldg(A.Tv + (oR * 4 + v) * N2 + tp);
-  if (PERT) {
-    r0L = (R)__ldg(A.bg.bgT + (oR * 2) * N2 + tp);
-    E0L = (R)__ldg(A.bg.bgT + (oR * 2 + 1) * N2 + tp);
-  }
   const Pt<R> sL = point_state<PERT>(qL, r0L, E0L, A.ph);
   const Pt<R> sR = point_state<PERT>(qR, r0R, E0R, A.ph);
   R Fh[5];
@@ -1123,6 +1126,7 @@ __device__ __forceinline__ void face_point(const KArgs<R>& A, const int2* __rest
 
 template <int N, bool PERT, class R>
 __global__ void __launch_bounds__(64) k_face(const KArgs<R> A, const int2* __restrict__ faces, int nf, int nw) {
+  pdl_trigger();
   face_point<N, PERT, R>(A, faces, nf, nw, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
 }
 
@@ -1158,6 +1162,11 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
     load_six(A.m.nbr, e, nbr);
     load_six(A.m.code, e, code);
   }
+  if (active) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) ij[i] = __ldg(A.m.invJ + (size_t)e * N3 + ln + N2 * i);
+  }
+  pdl_wait();
   const bool flagged = A.err != nullptr && (*(const volatile unsigned*)A.err & 1u) != 0;
   if (active) {
     const R* Fe = A.Fc + (size_t)e * 30 * N2 + ln;
@@ -1169,7 +1178,6 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int pt = ln + N2 * i;
-      ij[i] = __ldg(A.m.invJ + (size_t)e * N3 + pt);
 #pragma unroll
       for (int v = 0; v < 5; ++v) W[v][i] = A.out[((size_t)e * 5 + v) * N3 + pt];
     }
@@ -1229,15 +1237,40 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
 
 template <int N, class R, int EPB, int MODE>
 __global__ void __launch_bounds__(EPB * N * N) k_update(const KArgs<R> A) {
+  pdl_trigger();
   update_tile<N, R, EPB, MODE>(A, blockIdx.x);
 }
 
 // ------------------------------------------------------------------ launch helpers
 
+// Launch of a stage kernel that may start while the kernel before it on the stream drains (programmatic
+// dependent launch): every stage kernel lets its successor start at once (pdl_trigger) and reads what its
+// predecessor wrote only after pdl_wait, which returns once that kernel has completed and its writes are
+// visible.  A kernel completes only after its own wait, so the order reaches back along the stream.
+template <class... P, class... Q>
+cudaError_t launch_dependent(bool early, void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Q&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k, std::forward<Q>(args)...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <int N, bool PERT, class R, int EPB>
 struct Launch {
   static constexpr int threads = EPB * N * N;
   static int blocks(int E) { return (E + EPB - 1) / EPB; }
+  // Early launches (launch_dependent) pay where a stage is a few tens of microseconds: at 12,288 elements
+  // they took 8, 5, 4 and 1 % off a stage at p = 2..5 (p = 3, 288 elements: 23.1 -> 16.7 us), from 28,800
+  // they cost p = 2 and 3 1 to 9 % and the others gain nothing.
+  static bool early(int E) { return E <= 16384; }
 
   static cudaError_t trace(const MeshArg<R>& m, const OpsArg<R>& ops, const R* q, R* T, cudaStream_t st) {
     if (m.E == 0) return cudaSuccess;
@@ -1249,8 +1282,7 @@ struct Launch {
     if (A.Fc_out == nullptr || A.T == nullptr || A.Tv == nullptr) return cudaErrorInvalidValue;
     const int64_t n = (int64_t)(nf + nw) * N * N;
     // 64-thread CTAs (p = 3: 1 % faster than 128, 2.5 % faster than 256)
-    k_face<N, PERT, R><<<(unsigned)((n + 63) / 64), 64, 0, st>>>(A, faces, nf, nw);
-    return cudaGetLastError();
+    return launch_dependent(early(A.m.E), k_face<N, PERT, R>, (unsigned)((n + 63) / 64), 64, 0, st, A, faces, nf, nw);
   }
   template <int MODE>
   static cudaError_t vol(const KArgs<R>& A, cudaStream_t st) {
@@ -1270,8 +1302,7 @@ struct Launch {
     cudaError_t e =
         cudaFuncSetAttribute(k_vol<N, PERT, R, EPB, MODE, KR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_vol<N, PERT, R, EPB, MODE, KR><<<blocks(A.m.E), threads, sm, st>>>(A);
-    return cudaGetLastError();
+    return launch_dependent(early(A.m.E), k_vol<N, PERT, R, EPB, MODE, KR>, blocks(A.m.E), threads, sm, st, A);
   }
   template <int MODE>
   static cudaError_t update(const KArgs<R>& A, cudaStream_t st) {
@@ -1280,8 +1311,7 @@ struct Launch {
     const size_t sm = (size_t)UpLayout<N, R, EPB>::total * sizeof(R);
     cudaError_t e = cudaFuncSetAttribute(k_update<N, R, EPB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_update<N, R, EPB, MODE><<<blocks(A.m.E), threads, sm, st>>>(A);
-    return cudaGetLastError();
+    return launch_dependent(early(A.m.E), k_update<N, R, EPB, MODE>, blocks(A.m.E), threads, sm, st, A);
   }
 };
 
