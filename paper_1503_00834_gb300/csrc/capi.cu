@@ -35,12 +35,12 @@ template <class R>
 MeshArg<R> mesh_arg(const chorus_mesh_s* m);
 template <>
 MeshArg<double> mesh_arg<double>(const chorus_mesh_s* m) {
-  return MeshArg<double>{(int)m->E, m->d_nbr,   m->d_code, m->d_Sf64,
+  return MeshArg<double>{(int)m->E, m->d_nbr, m->d_code, m->d_fid, m->d_Sf64,
                          m->d_invJ64, m->d_x64, m->kr_active ? m->d_kr64 : nullptr, m->d_tab64, 0};
 }
 template <>
 MeshArg<float> mesh_arg<float>(const chorus_mesh_s* m) {
-  return MeshArg<float>{(int)m->E, m->d_nbr,   m->d_code, m->d_Sf32,
+  return MeshArg<float>{(int)m->E, m->d_nbr, m->d_code, m->d_fid, m->d_Sf32,
                         m->d_invJ32, m->d_g32, m->kr_active ? m->d_kr32 : nullptr, m->d_tab32, 0};
 }
 
@@ -447,6 +447,7 @@ void free_mesh(chorus_mesh_s* m) {
   free_background(m);
   dev_free(m->d_nbr);
   dev_free(m->d_code);
+  dev_free(m->d_fid);
   dev_free(m->d_Sf64);
   dev_free(m->d_invJ64);
   dev_free(m->d_x64);
@@ -616,7 +617,7 @@ chorus_status chorus_mesh_create(int64_t n_nodes, const double* node_xyz, int64_
           invJ[g] = 1.0 / m->host.detJ[g];
         }
   std::vector<float> f32(nS);
-  bool ok = dev_alloc(&m->d_nbr, E * 6) == cudaSuccess && dev_alloc(&m->d_code, E * 6) == cudaSuccess &&
+  bool ok = dev_alloc(&m->d_nbr, E * 6) == cudaSuccess && dev_alloc(&m->d_code, E * 6) == cudaSuccess && dev_alloc(&m->d_fid, E * 6) == cudaSuccess &&
             dev_alloc(&m->d_Sf64, nS) == cudaSuccess && dev_alloc(&m->d_invJ64, nP) == cudaSuccess &&
             dev_alloc(&m->d_x64, 3 * nP) == cudaSuccess && dev_alloc(&m->d_wJ, nP) == cudaSuccess &&
             dev_alloc(&m->d_Sf32, nS) == cudaSuccess && dev_alloc(&m->d_invJ32, nP) == cudaSuccess &&
@@ -638,6 +639,12 @@ chorus_status chorus_mesh_create(int64_t n_nodes, const double* node_xyz, int64_
     for (int F = 0; F < 6; ++F)
       if (m->host.nbr[e * 6 + F] < 0) faces.push_back(make_int2((int)e, F));
   m->n_wfaces = (int)faces.size() - m->n_ifaces;
+  std::vector<int> fid(E * 6);
+  for (size_t f = 0; f < faces.size(); ++f) {
+    const size_t own = (size_t)faces[f].x * 6 + faces[f].y;
+    fid[own] = (int)f;
+    if (m->host.nbr[own] >= 0) fid[(size_t)m->host.nbr[own] * 6 + (m->host.code[own] >> 3)] = (int)f;
+  }
   if (!faces.empty() && dev_alloc(&m->d_faces, faces.size()) != cudaSuccess) {
     free_mesh(m);
     return CHORUS_ENOMEM;
@@ -649,6 +656,7 @@ chorus_status chorus_mesh_create(int64_t n_nodes, const double* node_xyz, int64_
   };
   up(m->d_nbr, m->host.nbr.data(), E * 6 * sizeof(int));
   up(m->d_code, m->host.code.data(), E * 6 * sizeof(int));
+  up(m->d_fid, fid.data(), E * 6 * sizeof(int));
   up(m->d_Sf64, m->host.Sf.data(), nS * sizeof(double));
   up(m->d_invJ64, invJ.data(), nP * sizeof(double));
   up(m->d_x64, m->host.x.data(), 3 * nP * sizeof(double));
@@ -981,13 +989,14 @@ chorus_status run_rk(chorus_mesh_s* m, R* u, const Ws<R>& w, double dt, int64_t 
 constexpr int kHostChunks = 8;
 
 // The per-element arguments of the trace and update kernels shifted to elements [e0, e0 + ne): neither
-// reads neighbour data (the common face fluxes are in each element's own face numbering), so a range of
-// elements is a mesh of its own for them, but for the trace array, which they write as a whole.
+// reads the neighbours' elements, so a range of elements is a mesh of its own for them, but for the arrays
+// of the whole mesh's traces (written) and face fluxes (read).
 MeshArg<float> mesh_range(MeshArg<float> a, int64_t e0, int64_t ne, int N) {
   const int64_t N2 = N * N, N3 = N2 * N;
   a.E = (int)ne;
   a.nbr += e0 * 6;
   a.code += e0 * 6;
+  a.fid += e0 * 6;
   a.Sf += e0 * 9 * (N + 1) * N2;
   a.invJ += e0 * N3;
   a.x += e0 * 3 * N3;
@@ -1039,7 +1048,7 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
           RkCoef<float> ck = c;
           const int64_t o5 = e0 * 5 * N3;
           ck.out2 = c.out2 ? c.out2 + o5 : nullptr;
-          cudaError_t e = m->L.update32(mesh_range(ma, e0, ne, N), m->ops32, w.Fc + e0 * 30 * N2, dst + o5, Tn, ck, (float)dt, kModeRK, m->d_err, st);
+          cudaError_t e = m->L.update32(mesh_range(ma, e0, ne, N), m->ops32, w.Fc, dst + o5, Tn, ck, (float)dt, kModeRK, m->d_err, st);
           if (e == cudaSuccess) e = cudaEventRecord(m->copy_ev[k], st);
           if (e == cudaSuccess) e = cudaStreamWaitEvent(m->copy_stream, m->copy_ev[k], 0);
           if (e == cudaSuccess)

@@ -37,6 +37,7 @@ struct MeshArg {
   int E;
   const int* nbr;    // [E][6] neighbour element, -1 inner wall, -2 outer wall
   const int* code;   // [E][6] neighbour local face * 8 + orientation bits
+  const int* fid;    // [E][6] position of the face in the face list
   const R* Sf;       // [E][3 d][3 n][N+1 f][N*N line]  S^d_n = |J| d xi_d / d x_n at the d-flux points
   const R* invJ;     // [E][N^3] 1/|J| at the solution points
   const R* x;        // [E][3][N^3] solution-point coordinates x; FP32: x / |x|^3 (gravity)
@@ -86,8 +87,8 @@ struct RkCoef {
 //   trace   face traces of q, each in the neighbour's slot (trace_slot); T: of the whole mesh
 //   vol     from q and its traces: one-sided viscous face fluxes Tv and `out`, the residual (mode
 //           kModeResidual) or stage state (kModeRK, and rk.out2) without the end-point fluxes; `out` may be q
-//   face    common face fluxes F~ [E][6][5][N^2] of the face list (n_faces interior faces, from their
-//           lower element, then n_walls wall faces)
+//   face    common fluxes Fc [faces][5][N^2], along the owner's outward S, of the face list (n_faces
+//           interior faces, from their lower element, then n_walls wall faces)
 //   update  the end-point fluxes' part added to `out` (and rk.out2); T_out: traces of the new state
 //           (of the whole mesh)
 struct LaunchSet {

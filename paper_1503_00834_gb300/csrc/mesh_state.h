@@ -25,6 +25,7 @@ struct chorus_mesh_s {
   // device mesh arrays
   int* d_nbr = nullptr;
   int* d_code = nullptr;
+  int* d_fid = nullptr;
   double* d_Sf64 = nullptr;
   double* d_invJ64 = nullptr;
   double* d_x64 = nullptr;
