@@ -195,7 +195,8 @@ chorus_status persist_rk3_step(StagePtrs* const groups[4], double dt, unsigned* 
       KArgs<float>& f = P.face[s];
       f.m = G.m; f.ph = G.ph; f.bg = G.bg; f.T = Tc; f.Tv = G.Tv; f.Fc_out = G.Fc; f.err = err;
       KArgs<float>& r = P.update[s];
-      r.m = G.m; r.ops = G.ops; r.Fc = G.Fc; r.out = G.buf[sg.dst]; r.T_out = Tn; r.c = (float)sg.c;
+      r.m = G.m; r.ops = G.ops; r.Fc = G.Fc; r.out = G.buf[sg.dst]; r.T_out = k + 1 < (int)stg.size() ? Tn : nullptr;
+      r.c = (float)sg.c;
       r.dt = (float)dt; r.err = err;
       P.faces[s] = G.faces;
       P.nf[s] = G.nf;
