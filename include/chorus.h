@@ -392,7 +392,8 @@ chorus_status chorus_batch_autotune(chorus_batch batch, float* Q, void* workspac
 
 /* Schedule of the orders within a batch step: set 1 = concurrent streams, 0 = one after another,
  * 2 = one persistent launch per RK stage (CHORUS_EUNSUPPORTED without cooperative launch or with a
- * radial kappa_r(r)), any other value leaves it; concurrent: host int receiving the schedule in
+ * radial kappa_r(r)), any other value leaves it (a new batch: concurrent below 2^20 solution points,
+ * else one after another); concurrent: host int receiving the schedule in
  * force (0, 1 or 2), or NULL. */
 chorus_status chorus_batch_schedule(chorus_batch batch, int set, int* concurrent);
 
