@@ -75,7 +75,8 @@ def kernel_sources_digest() -> str:
     import re
 
     csrc = os.path.join(ROOT, "paper_1503_00834_gb300", "csrc")
-    names = ["internal.h", "sd_device.cuh", "sd_kernels.cuh", "kern_inst.cuh"] + [f"kern_p{p}.cu" for p in (2, 3, 4, 5)]
+    names = ["internal.h", "sd_device.cuh", "sd_physics.cuh", "sd_kernels.cuh", "kern_inst.cuh"]
+    names += [f"kern_p{p}.cu" for p in (2, 3, 4, 5)]
     names.append(os.path.join("..", "build.py"))
     h = hashlib.sha256()
     for n in names:

@@ -321,8 +321,8 @@ chorus_status chorus_residual_noalloc(chorus_mesh mesh, const chorus_params* par
  *    stage is one launch per order present; the orders run concurrently on forked streams or one
  *    after another, and one RK step of the whole batch is captured once as a CUDA graph and
  *    replayed.  A third schedule runs every order in one persistent cooperative launch per RK
- *    stage: its CTAs take (order, tile) work items of each phase (traces, lifting, face fluxes,
- *    residual; the orders' tiles in one list) from a counter and meet at bounded grid barriers
+ *    stage: its CTAs take (order, tile) work items of each phase (traces, volume, face fluxes,
+ *    update; the orders' tiles in one list) from a counter and meet at bounded grid barriers
  *    between the phases (a barrier that runs out of polls sets CHORUS_ETIMEOUT; nothing spins
  *    unbounded).  chorus_batch_schedule sets it; the autotuner times all three.
  *  - State: FP32 perturbation form (CHORUS_FP32_PERT) only.  One caller-owned device array holds

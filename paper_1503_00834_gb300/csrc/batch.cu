@@ -290,7 +290,7 @@ chorus_status chorus_batch_init(chorus_batch b, float* Q, void* stream) {
 chorus_status chorus_batch_rk_step(chorus_batch b, float* Q, void* workspace, double dt, int64_t n_steps,
                                    void* stream, int64_t* launches) {
   if (!b || !Q || !workspace || !(dt > 0.0) || !std::isfinite(dt) || n_steps < 0) return CHORUS_EINVAL;
-  // per order: trace + 3 x (gradient, face, residual); persistent: one launch per stage
+  // per order: trace + 3 x (volume, face, update); persistent: one launch per stage
   if (launches) *launches = b->persistent ? 3 : 10 * (int64_t)b->groups.size();
   if (n_steps == 0) return CHORUS_OK;
   cudaStream_t st = (cudaStream_t)stream;

@@ -1,7 +1,7 @@
 // The three-pass kernels of the FP32 SSP-RK(5,4) stages (chorus_rk_step_scheme, scheme 1) and of the FP64
 // residual of the background that chorus_prepare takes the FP32 tables from: lifting with the
 // gradient record written to global memory (k_grad), common face fluxes (k_face), fluxes, update and
-// traces (k_resid).  The two-kernel form of sd_kernels.cuh is 1.2 to 2 times faster a stage but rounds
+// traces (k_resid).  The form of sd_kernels.cuh is 1.2 to 2 times faster a stage but rounds
 // the FP32 sums in another order.  The paper's integrator is what production runs step with, followed by
 // chorus_am_correct, whose FP64 rates delta Omega are integrals that cancel down to the state's FP32
 // rounding: another rounding of the stages changes them by 1e-7 relative on the first step and by 2e-4
