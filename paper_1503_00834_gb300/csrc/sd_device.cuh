@@ -46,6 +46,20 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Load of a value that another kernel, or another phase of the same launch, has written since this kernel
+// started.  __ldg is for data that no one writes while the kernel runs: the compiler may move it above
+// pdl_wait or a grid barrier, and its cache line may be stale.  The volatile asm keeps its place.
+__device__ __forceinline__ float ld_written(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_written(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+
 // Polls of a bounded mbarrier wait when the mesh sets no limit of its own (about a second with the
 // back-off below).
 constexpr uint32_t kDefaultWaitPolls = 1u << 24;

@@ -209,7 +209,7 @@ __device__ __forceinline__ void lift_prefetch(const KArgs<R>& A, int e, int ln, 
     const R* Te = A.T + ((size_t)e * 6 + 2 * D + side) * 5 * N2 + ln;
     p.nb[side].kind = nbr[2 * D + side];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) p.nb[side].q[v] = __ldg(Te + v * N2);
+    for (int v = 0; v < 5; ++v) p.nb[side].q[v] = ld_written(Te + v * N2);
   }
 }
 
@@ -1027,7 +1027,7 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
         R Rv = -(x.g[(kG + v) * N3 + si] + acc[v][i]) * cur.ij - M[v];
         if (PERT) Rv += cur.r0[v];
         const size_t oi = ((size_t)e * 5 + v) * N3 + pt;
-        if (decltype(extra)::value && A.radd) Rv += __ldg(A.radd + oi);
+        if (decltype(extra)::value && A.radd) Rv += ld_written(A.radd + oi);
         if (MODE == kModeResidual) {
           A.out[oi] = Rv;
         } else {
@@ -1095,9 +1095,9 @@ __device__ __forceinline__ void face_point(const KArgs<R>& A, const int2* __rest
   }
   pdl_wait();
 #pragma unroll
-  for (int v = 0; v < 5; ++v) qR[v] = __ldg(A.T + (oL * 5 + v) * N2 + t);
+  for (int v = 0; v < 5; ++v) qR[v] = ld_written(A.T + (oL * 5 + v) * N2 + t);
 #pragma unroll
-  for (int v = 0; v < 4; ++v) tvL[v] = __ldg(A.Tv + (oL * 4 + v) * N2 + t);
+  for (int v = 0; v < 4; ++v) tvL[v] = ld_written(A.Tv + (oL * 4 + v) * N2 + t);
   if (wall) {  // exact inviscid flux (0, p S, 0) minus the normal viscous traction; energy: f.S
     const Pt<R> st = point_state<PERT>(qR, r0R, E0R, A.ph);
     const R mag2 = dot3(So, So);
@@ -1109,9 +1109,9 @@ __device__ __forceinline__ void face_point(const KArgs<R>& A, const int2* __rest
     return;
   }
 #pragma unroll
-  for (int v = 0; v < 5; ++v) qL[v] = __ldg(A.T + (oR * 5 + v) * N2 + tp);
+  for (int v = 0; v < 5; ++v) qL[v] = ld_written(A.T + (oR * 5 + v) * N2 + tp);
 #pragma unroll
-  for (int v = 0; v < 4; ++v) tvR[v] = __ldg(A.Tv + (oR * 4 + v) * N2 + tp);
+  for (int v = 0; v < 4; ++v) tvR[v] = ld_written(A.Tv + (oR * 4 + v) * N2 + tp);
   const Pt<R> sL = point_state<PERT>(qL, r0L, E0L, A.ph);
   const Pt<R> sR = point_state<PERT>(qR, r0R, E0R, A.ph);
   R Fh[5];
@@ -1175,7 +1175,7 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
       const R sg = own == ((F & 1) != 0) ? R(1) : R(-1);
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const R f = sg * __ldg(Ff + v * N2);
+        const R f = sg * ld_written(Ff + v * N2);
         if (F < 4) Fxy[F < 4 ? 5 * F + v : 0] = f;
         else Fz[F < 4 ? 0 : F - 4][v] = f;
       }
