@@ -21,8 +21,11 @@ constexpr int kPMinBlocks = 3;     // resident CTAs per SM asked of the compiler
 template <int S>
 __host__ __device__ constexpr int p_epb() { return S == 0 ? 14 : S == 1 ? 8 : S == 2 ? 5 : 3; }
 
-// staging barriers of a CTA: p = 3 tiles stage by warps (unit_elems), the others by the CTA
-constexpr int kPBars = kVolBars * (kPThreads / 32);
+// barriers of a CTA, a set for each order: p = 3 tiles stage by warps (unit_elems), the others by the CTA
+__host__ __device__ constexpr int bar_offset(int slot) {
+  return kVolBars * (slot + (slot > 1 ? kPThreads / 32 - 1 : 0));
+}
+constexpr int kPBars = bar_offset(4);
 
 struct PersistArgs {
   KArgs<float> vol[4], face[4], update[4];  // slot p - 2; an absent order has no work items
@@ -84,8 +87,13 @@ template <int S>
 __device__ __noinline__ void update_item(const PersistArgs& P, int64_t t) {
   update_tile<S + 3, float, p_epb<S>(), kModeRK>(P.update[S], t);
 }
+// Each order has barriers and a parity of its own: the orders use different numbers of them (a warp's
+// own at N = 4, the staging's alone at N = 5 and 6), so after an item of one order another order's
+// barriers have not completed the same number of phases.
 template <int S>
-__device__ __forceinline__ void run_item(const PersistArgs& P, int phase, int64_t t, uint64_t* bar, uint32_t& pbar) {
+__device__ __forceinline__ void run_item(const PersistArgs& P, int phase, int64_t t, uint64_t* bars, uint32_t (&par)[4]) {
+  uint64_t* bar = bars + bar_offset(S);
+  uint32_t& pbar = par[S];
   if (phase == 0) trace_item<S>(P, t);
   else if (phase == 1) vol_item<S>(P, t, bar, pbar);
   else if (phase == 2) face_item<S>(P, t);
@@ -101,7 +109,7 @@ __global__ void __launch_bounds__(kPThreads, kPMinBlocks) k_batch_stage(const __
     s_stop = 0;
   }
   __syncthreads();
-  uint32_t pbar = 0;
+  uint32_t pbar[4] = {0, 0, 0, 0};
   unsigned barriers = 0;
   const uint32_t polls = wait_polls(P.err);  // the grid barriers' limit: the staging waits' own
   for (int phase = P.trace ? 0 : 1; phase < 4; ++phase) {
@@ -123,6 +131,7 @@ __global__ void __launch_bounds__(kPThreads, kPMinBlocks) k_batch_stage(const __
       else if (slot == 2) run_item<2>(P, phase, t, bar, pbar);
       else if (slot == 1) run_item<1>(P, phase, t, bar, pbar);
       else run_item<0>(P, phase, t, bar, pbar);
+      fence_async_smem();  // before the next tile's bulk copies
       __syncthreads();  // the tile's shared memory is free for the next one
       if (threadIdx.x == 0 && (*(volatile unsigned*)P.err & 1u)) s_stop = 1;  // a bounded wait gave up
     }
