@@ -213,7 +213,7 @@ chorus_status chorus_am_correct(chorus_mesh mesh, const chorus_params* params, c
  * 135 -> 128 (SiLU) -> 128 (SiLU) -> 135; its output times out_scale[v] is added to dQ/dt.
  * Record (device, caller-owned, chorus_closure_bytes() bytes): BF16 W1 [128][135], W2 [128][128],
  * W3 [135][128] (row-major, output index first), FP32 b1 [128], b2 [128], b3 [135], in_scale [5],
- * out_scale [5].  Arithmetic accumulates in FP32. */
+ * out_scale [5].  The record's address is a multiple of 4.  Arithmetic accumulates in FP32. */
 size_t chorus_closure_bytes(void);
 
 /* Seeded initial record: weights uniform in +-sqrt(3/fan_in) (output layer x 0.1), zero biases,

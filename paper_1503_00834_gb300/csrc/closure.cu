@@ -215,14 +215,26 @@ __device__ __forceinline__ void stage_w1(const __nv_bfloat16* __restrict__ Wg, _
       reinterpret_cast<unsigned short*>(sW)[c * SW1 + k] = k < NI ? __ldg(src + c * NI + k) : (unsigned short)0;
 }
 
-// W2 or W3 ([ROWS][NH], a warp a row) at row stride SW2; a zero row after an odd number of rows.
+// W2 or W3 ([ROWS][NH], a warp a row) at row stride SW2; a zero row after an odd number of rows.  The
+// record needs the 4-byte alignment of its FP32 fields only: rows that do not start on an 8-byte boundary
+// (the same for all of a matrix) are read in 4-byte halves.
 template <int TB, int ROWS>
 __device__ __forceinline__ void stage_w(const __nv_bfloat16* __restrict__ Wg, __nv_bfloat16* sW) {
   static_assert(ClosureLayout::oW2 % 8 == 0 && ClosureLayout::oW3 % 8 == 0 && NH == 128, "rows of 32 8-byte units");
   const int lane = threadIdx.x & 31;
-  for (int c = threadIdx.x >> 5; c < ROWS + ROWS % 2; c += TB / 4)
-    *reinterpret_cast<uint2*>(sW + c * SW2 + 4 * lane) =
-        c < ROWS ? __ldg(reinterpret_cast<const uint2*>(Wg + c * NH) + lane) : make_uint2(0u, 0u);
+  const bool v8 = ((uintptr_t)Wg & 7u) == 0;
+  for (int c = threadIdx.x >> 5; c < ROWS + ROWS % 2; c += TB / 4) {
+    uint2 v = make_uint2(0u, 0u);
+    if (c < ROWS) {
+      if (v8) {
+        v = __ldg(reinterpret_cast<const uint2*>(Wg + c * NH) + lane);
+      } else {
+        const unsigned* h = reinterpret_cast<const unsigned*>(Wg + c * NH) + 2 * lane;
+        v = make_uint2(__ldg(h), __ldg(h + 1));
+      }
+    }
+    *reinterpret_cast<uint2*>(sW + c * SW2 + 4 * lane) = v;
+  }
 }
 
 __device__ __forceinline__ void bf16x4(const __nv_bfloat16* p, float w[4]) {
