@@ -415,11 +415,13 @@ chorus_status chorus_set_well_balanced(chorus_mesh mesh, int enable);
  * mesh's kernels, then clear it. */
 chorus_status chorus_check(chorus_mesh mesh, void* stream);
 
-/* Limit of the bounded device-side waits with which the volume kernel of this mesh waits for the bulk
- * copies that stage each element's state, background and metrics in shared memory: after `polls` polls
- * the wait gives up, the kernel sets the mesh's error flag, waits (with the default limit) for its
- * copies still in flight and returns without storing its elements, and while the flag is set the kernel
- * that completes the residual or stage leaves it as it is; chorus_check then reports CHORUS_ETIMEOUT.  polls < 0 restores the default (2^24 polls
+/* Limit of the bounded device-side waits with which the kernels of this mesh (the volume kernel; in the
+ * FP32 SSP-RK(5,4) stages the lifting and residual kernels) wait for the bulk copies that stage each
+ * element's arrays in shared memory: after `polls` polls the wait gives up, the kernel sets the mesh's
+ * error flag, waits (with the default limit) for its copies still in flight and returns without storing its
+ * elements, and the kernel that completes the residual or stage leaves those elements as they are;
+ * chorus_check then reports CHORUS_ETIMEOUT.  The flag holds up no later call: one whose waits are met is
+ * complete whether or not the flag has been read.  polls < 0 restores the default (2^24 polls
  * with back-off, about a second); 0 makes every wait give up at once, so the failure path can be
  * exercised without a fault.  polls >= 2^32 - 1: CHORUS_EINVAL.  Synchronous. */
 chorus_status chorus_set_wait_limit(chorus_mesh mesh, int64_t polls);

@@ -113,6 +113,9 @@ __global__ void __launch_bounds__(kPThreads, kPMinBlocks) k_batch_stage(const __
   unsigned barriers = 0;
   const uint32_t polls = wait_polls(P.err);  // the grid barriers' limit: the staging waits' own
   for (int phase = P.trace ? 0 : 1; phase < 4; ++phase) {
+    // a wait that gave up before the phase: not even the first item (the volume phase may have stopped
+    // before every element, so the update phase must not run)
+    if (threadIdx.x == 0 && (*(volatile unsigned*)P.err & 1u)) s_stop = 1;
     const int64_t total = P.items[phase][0] + P.items[phase][1] + P.items[phase][2] + P.items[phase][3];
     for (;;) {
       if (threadIdx.x == 0) s_item = atomicAdd(P.sync + 1 + phase, 1u);
@@ -200,13 +203,13 @@ chorus_status persist_rk3_step(StagePtrs* const groups[4], double dt, unsigned* 
       KArgs<float>& a = P.vol[s];
       a.m = G.m; a.ops = G.ops; a.ph = G.ph; a.bg = G.bg; a.q = G.buf[sg.src]; a.T = Tc; a.Tv_out = G.Tv;
       a.out = G.buf[sg.dst]; a.un = G.buf[sg.un]; a.a = (float)sg.a; a.b = (float)sg.b; a.c = (float)sg.c;
-      a.dt = (float)dt; a.err = err;
+      a.dt = (float)dt; a.skip_out = G.skip; a.err = err;
       KArgs<float>& f = P.face[s];
       f.m = G.m; f.ph = G.ph; f.bg = G.bg; f.T = Tc; f.Tv = G.Tv; f.Fc_out = G.Fc; f.err = err;
       KArgs<float>& r = P.update[s];
       r.m = G.m; r.ops = G.ops; r.Fc = G.Fc; r.out = G.buf[sg.dst]; r.T_out = k + 1 < (int)stg.size() ? Tn : nullptr;
       r.c = (float)sg.c;
-      r.dt = (float)dt; r.err = err;
+      r.dt = (float)dt; r.skip = G.skip;
       P.faces[s] = G.faces;
       P.nf[s] = G.nf;
       P.nw[s] = G.nw;

@@ -484,6 +484,7 @@ struct Ws {
   R* B;
   R* G;
   R* Fc;
+  int* skip;  // [E] in G, which the stage kernels that use the marks leave alone
 };
 
 template <class R>
@@ -500,6 +501,7 @@ Ws<R> split_ws(const chorus_mesh_s* m, void* w) {
   r.B = r.A + E * 5 * N3;
   r.G = r.B + E * 5 * N3;
   r.Fc = r.G + E * 12 * N3;
+  r.skip = (int*)r.G;
   return r;
 }
 
@@ -901,11 +903,11 @@ chorus_status chorus_residual(chorus_mesh m, const chorus_params* P, chorus_prec
     CHK(timed(m, 0, st, [&] { return m->L.trace64(ma, m->ops64, (const double*)Q, w.Ta, st); }));
     CHK(timed(m, 1, st, [&] {
       return m->L.vol64(ma, m->ops64, ph, (const double*)Q, w.Ta, w.Tv, (double*)R, rc, 0.0, kModeResidual,
-                        m->d_err, st);
+                         w.skip, m->d_err, st);
     }));
     CHK(timed(m, 3, st, [&] { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
     CHK(timed(m, 2, st, [&] {
-      return m->L.update64(ma, m->ops64, w.Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, m->d_err, st);
+      return m->L.update64(ma, m->ops64, w.Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, w.skip, st);
     }));
     return CHORUS_OK;
   }
@@ -924,12 +926,12 @@ chorus_status chorus_residual(chorus_mesh m, const chorus_params* P, chorus_prec
   }
   CHK(timed(m, 0, st, [&] { return m->L.trace32(ma, m->ops32, (const float*)Q, w.Ta, st); }));
   CHK(timed(m, 1, st, [&] {
-    return m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, (float*)R, rc, 0.0f, kModeResidual, m->d_err,
-                      st);
+    return m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, (float*)R, rc, 0.0f, kModeResidual,
+                       w.skip, m->d_err, st);
   }));
   CHK(timed(m, 3, st, [&] { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
   CHK(timed(m, 2, st, [&] {
-    return m->L.update32(ma, m->ops32, w.Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, m->d_err, st);
+    return m->L.update32(ma, m->ops32, w.Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, w.skip, st);
   }));
   return CHORUS_OK;
 }
@@ -1037,12 +1039,12 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
   const chorus_status s = run_rk<float>(
       m, Qd, w, dt, n_steps, 0, st,
       [&](const float* q, const float* T, float* dst, const RkCoef<float>& c) {
-        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, dst, c, (float)dt, kModeRK, m->d_err, st);
+        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, dst, c, (float)dt, kModeRK, w.skip, m->d_err, st);
       },
       [&](const float* T) { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
       [&](float* dst, float* Tn, const RkCoef<float>& c) -> cudaError_t {
         if (++stage < last || dst != Qd)
-          return m->L.update32(ma, m->ops32, w.Fc, dst, Tn, c, (float)dt, kModeRK, m->d_err, st);
+          return m->L.update32(ma, m->ops32, w.Fc, dst, Tn, c, (float)dt, kModeRK, w.skip, st);
         for (int k = 0; k < kHostChunks; ++k) {
           int64_t e0, ne;
           range(k, &e0, &ne);
@@ -1050,7 +1052,8 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
           RkCoef<float> ck = c;
           const int64_t o5 = e0 * 5 * N3;
           ck.out2 = c.out2 ? c.out2 + o5 : nullptr;
-          cudaError_t e = m->L.update32(mesh_range(ma, e0, ne, N), m->ops32, w.Fc, dst + o5, Tn, ck, (float)dt, kModeRK, m->d_err, st);
+          cudaError_t e = m->L.update32(mesh_range(ma, e0, ne, N), m->ops32, w.Fc, dst + o5, Tn, ck, (float)dt, kModeRK,
+                                          w.skip + e0, st);
           if (e == cudaSuccess) e = cudaEventRecord(m->copy_ev[k], st);
           if (e == cudaSuccess) e = cudaStreamWaitEvent(m->copy_stream, m->copy_ev[k], 0);
           if (e == cudaSuccess)
@@ -1144,11 +1147,11 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
     return run_rk<double>(
         m, (double*)Q, w, dt, n_steps, scheme, st,
         [&](const double* q, const double* T, double* dst, const RkCoef<double>& c) {
-          return m->L.vol64(ma, m->ops64, ph, q, T, w.Tv, dst, c, dt, kModeRK, m->d_err, st);
+          return m->L.vol64(ma, m->ops64, ph, q, T, w.Tv, dst, c, dt, kModeRK, w.skip, m->d_err, st);
         },
         [&](const double* T) { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
         [&](double* dst, double* Tn, const RkCoef<double>& c) {
-          return m->L.update64(ma, m->ops64, w.Fc, dst, Tn, c, dt, kModeRK, m->d_err, st);
+          return m->L.update64(ma, m->ops64, w.Fc, dst, Tn, c, dt, kModeRK, w.skip, st);
         },
         [&](const double* q, double* T) { return m->L.trace64(ma, m->ops64, q, T, st); });
   }
@@ -1181,11 +1184,11 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
   return run_rk<float>(
       m, (float*)Q, w, dt, n_steps, scheme, st,
       [&](const float* q, const float* T, float* dst, const RkCoef<float>& c) {
-        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, dst, c, (float)dt, kModeRK, m->d_err, st);
+        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, dst, c, (float)dt, kModeRK, w.skip, m->d_err, st);
       },
       [&](const float* T) { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
       [&](float* dst, float* Tn, const RkCoef<float>& c) {
-        return m->L.update32(ma, m->ops32, w.Fc, dst, Tn, c, (float)dt, kModeRK, m->d_err, st);
+        return m->L.update32(ma, m->ops32, w.Fc, dst, Tn, c, (float)dt, kModeRK, w.skip, st);
       },
       [&](const float* q, float* T) { return m->L.trace32(ma, m->ops32, q, T, st); });
 }
@@ -1566,7 +1569,7 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
   const size_t word = prec == CHORUS_FP64 ? sizeof(double) : sizeof(float);
   const size_t N3 = N2 * (size_t)m->N;
   const size_t nT = E * 6 * 5 * N2, nTv = E * 6 * 4 * N2;
-  // the documented size limit (more than the traces and the two face-flux arrays need today)
+  // the documented size limit (more than the traces, the two face-flux arrays and the marks need today)
   if ((2 * nT + nTv + E * 12 * N3) * word > kNoAllocScratchBytes) return CHORUS_EINVAL;  // mesh too large for the scratch
   if (prec == CHORUS_FP32_PERT && (!m->prepared || !same_params(m->prep, *P))) return CHORUS_EINVAL;
   // the attached closure's output buffer was allocated by chorus_closure_attach; FP64 reads Q0
@@ -1585,15 +1588,16 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
     double* T = (double*)scratch;
     double* Tv = T + nT;
     double* Fc = Tv + nTv;
+    int* skip = (int*)(Fc + nT);
     RkCoef<double> rc{};
     if (m->closure) {
       CHK(mlp_elements_tc(0, m->closure, Q, m->d_Q0, m->closure_buf, m->E, 0, m->d_err, st));
       rc.radd = (const double*)m->closure_buf;
     }
     CHK(m->L.trace64(ma, m->ops64, (const double*)Q, T, st));
-    CHK(m->L.vol64(ma, m->ops64, ph, (const double*)Q, T, Tv, (double*)R, rc, 0.0, kModeResidual, m->d_err, st));
+    CHK(m->L.vol64(ma, m->ops64, ph, (const double*)Q, T, Tv, (double*)R, rc, 0.0, kModeResidual, skip, m->d_err, st));
     CHK(m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st));
-    CHK(m->L.update64(ma, m->ops64, Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, m->d_err, st));
+    CHK(m->L.update64(ma, m->ops64, Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, skip, st));
     return CHORUS_OK;
   }
   const PhysArg<float> ph = phys_arg<float>(*P, m->r_inner, m->r_outer);
@@ -1602,15 +1606,16 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
   float* T = (float*)scratch;
   float* Tv = T + nT;
   float* Fc = Tv + nTv;
+  int* skip = (int*)(Fc + nT);
   RkCoef<float> rc{};
   if (m->closure) {
     CHK(mlp_elements_tc(1, m->closure, Q, nullptr, m->closure_buf, m->E, 0, m->d_err, st));
     rc.radd = (const float*)m->closure_buf;
   }
   CHK(m->L.trace32(ma, m->ops32, (const float*)Q, T, st));
-  CHK(m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, (float*)R, rc, 0.0f, kModeResidual, m->d_err, st));
+  CHK(m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, (float*)R, rc, 0.0f, kModeResidual, skip, m->d_err, st));
   CHK(m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st));
-  CHK(m->L.update32(ma, m->ops32, Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, m->d_err, st));
+  CHK(m->L.update32(ma, m->ops32, Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, skip, st));
   return CHORUS_OK;
 }
 
@@ -1674,6 +1679,7 @@ chorus_status mesh_stage_ptrs(chorus_mesh_s* m, const chorus_params& P, float* u
   out->Tb = w.Tb;
   out->Tv = w.Tv;
   out->Fc = w.Fc;
+  out->skip = w.skip;
   out->faces = m->d_faces;
   out->nf = m->n_ifaces;
   out->nw = m->n_wfaces;

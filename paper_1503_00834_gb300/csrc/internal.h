@@ -91,23 +91,25 @@ struct RkCoef {
 //           interior faces, from their lower element, then n_walls wall faces)
 //   update  the end-point fluxes' part added to `out` (and rk.out2); T_out: traces of the new state
 //           (of the whole mesh)
+// skip [E]: vol marks the elements whose staging gave up (it stores nothing for them), update leaves
+// those as they are.
 struct LaunchSet {
   cudaError_t (*trace64)(const MeshArg<double>&, const OpsArg<double>&, const double* q, double* T, cudaStream_t);
   cudaError_t (*vol64)(const MeshArg<double>&, const OpsArg<double>&, const PhysArg<double>&, const double* q,
                        const double* T, double* Tv, double* out, const RkCoef<double>& rk,
-                       double dt, int mode, unsigned* err, cudaStream_t);
+                       double dt, int mode, int* skip, unsigned* err, cudaStream_t);
   cudaError_t (*face64)(const MeshArg<double>&, const PhysArg<double>&, const int2* faces, int n_faces, int n_walls,
                         const double* T, const double* Tv, double* Fc, cudaStream_t);
   cudaError_t (*update64)(const MeshArg<double>&, const OpsArg<double>&, const double* Fc, double* out, double* T_out,
-                          const RkCoef<double>& rk, double dt, int mode, unsigned* err, cudaStream_t);
+                          const RkCoef<double>& rk, double dt, int mode, const int* skip, cudaStream_t);
   cudaError_t (*trace32)(const MeshArg<float>&, const OpsArg<float>&, const float* q, float* T, cudaStream_t);
   cudaError_t (*vol32)(const MeshArg<float>&, const OpsArg<float>&, const PhysArg<float>&, const BgArg&,
                        const float* q, const float* T, float* Tv, float* out, const RkCoef<float>& rk, float dt,
-                       int mode, unsigned* err, cudaStream_t);
+                       int mode, int* skip, unsigned* err, cudaStream_t);
   cudaError_t (*face32)(const MeshArg<float>&, const PhysArg<float>&, const BgArg&, const int2* faces, int n_faces,
                         int n_walls, const float* T, const float* Tv, float* Fc, cudaStream_t);
   cudaError_t (*update32)(const MeshArg<float>&, const OpsArg<float>&, const float* Fc, float* out, float* T_out,
-                          const RkCoef<float>& rk, float dt, int mode, unsigned* err, cudaStream_t);
+                          const RkCoef<float>& rk, float dt, int mode, const int* skip, cudaStream_t);
   int epb32;  // elements per CTA of the FP32 volume kernel
 };
 

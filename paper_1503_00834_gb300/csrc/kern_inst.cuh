@@ -20,22 +20,22 @@ struct Inst {
   }
   static cudaError_t vol64(const MeshArg<double>& m, const OpsArg<double>& ops, const PhysArg<double>& ph,
                            const double* q, const double* T, double* Tv, double* out,
-                           const RkCoef<double>& rk, double dt, int mode, unsigned* err, cudaStream_t st) {
+                           const RkCoef<double>& rk, double dt, int mode, int* skip, unsigned* err, cudaStream_t st) {
     using L = Launch<N, false, double, EPB64>;
     KArgs<double> A{};
     A.m = m; A.ops = ops; A.ph = ph; A.q = q; A.T = T; A.Tv_out = Tv; A.out = out;
     set_rk(A, rk);
-    A.dt = dt; A.err = err;
+    A.dt = dt; A.skip_out = skip; A.err = err;
     return mode == kModeRK ? L::template vol<kModeRK>(A, st) : L::template vol<kModeResidual>(A, st);
   }
   static cudaError_t vol32(const MeshArg<float>& m, const OpsArg<float>& ops, const PhysArg<float>& ph,
                            const BgArg& bg, const float* q, const float* T, float* Tv, float* out,
-                           const RkCoef<float>& rk, float dt, int mode, unsigned* err, cudaStream_t st) {
+                           const RkCoef<float>& rk, float dt, int mode, int* skip, unsigned* err, cudaStream_t st) {
     using L = Launch<N, true, float, EPB32>;
     KArgs<float> A{};
     A.m = m; A.ops = ops; A.ph = ph; A.bg = bg; A.q = q; A.T = T; A.Tv_out = Tv; A.out = out;
     set_rk(A, rk);
-    A.dt = dt; A.err = err;
+    A.dt = dt; A.skip_out = skip; A.err = err;
     return mode == kModeRK ? L::template vol<kModeRK>(A, st) : L::template vol<kModeResidual>(A, st);
   }
   static cudaError_t face64(const MeshArg<double>& m, const PhysArg<double>& ph, const int2* faces, int nf, int nw,
@@ -52,12 +52,12 @@ struct Inst {
   }
   template <bool PERT, class R, int EPB>
   static cudaError_t update(const MeshArg<R>& m, const OpsArg<R>& ops, const R* Fc, R* out, R* T_out,
-                            const RkCoef<R>& rk, R dt, int mode, unsigned* err, cudaStream_t st) {
+                            const RkCoef<R>& rk, R dt, int mode, const int* skip, cudaStream_t st) {
     using L = Launch<N, PERT, R, EPB>;
     KArgs<R> A{};
     A.m = m; A.ops = ops; A.Fc = Fc; A.out = out; A.T_out = T_out;
     set_rk(A, rk);
-    A.dt = dt; A.err = err;
+    A.dt = dt; A.skip = skip;
     return mode == kModeRK ? L::template update<kModeRK>(A, st) : L::template update<kModeResidual>(A, st);
   }
   static LaunchSet set() {

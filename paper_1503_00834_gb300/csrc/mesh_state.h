@@ -109,6 +109,7 @@ struct StagePtrs {
   BgArg bg;
   float* buf[4];  // stage buffers: u, s, A, B (ids of Stage)
   float *Ta, *Tb, *Tv, *Fc;
+  int* skip;
   const int2* faces;
   int nf, nw;
   unsigned* err;

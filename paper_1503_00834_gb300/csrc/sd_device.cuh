@@ -54,6 +54,11 @@ __device__ __forceinline__ float ld_written(const float* p) {
   asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
 }
+__device__ __forceinline__ int ld_written(const int* p) {
+  int v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
 __device__ __forceinline__ double ld_written(const double* p) {
   double v;
   asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));

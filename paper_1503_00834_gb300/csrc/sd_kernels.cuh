@@ -147,7 +147,9 @@ struct KArgs {
   const R* radd;       // optional additive residual correction [E][5][N3]
   R* Fc_out;           // k_face output: common fluxes along the owner's outward S [faces][5][N2]
   const R* Fc;         // k_update input
-  unsigned* err;
+  int* skip_out;       // k_vol: per element, 1 if its staging gave up (nothing stored for it), else 0
+  const int* skip;     // k_update: the same; elements with 1 are left as they are
+  unsigned* err;       // k_vol: error flags and wait limit
 };
 
 // Face traces are kept where they are read: slot (e, F) of a trace array holds, at element e's own
@@ -889,8 +891,10 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
           lift_prefetch<N, R, 1, L::SM>(A, e, ln, pre[1], nbr);
           lift_prefetch<N, R, 0, L::SM>(A, e, ln, pre[2], nbr);
         }
-      }))
+      })) {
+    if (active && ln == 0) A.skip_out[e] = 1;
     return;
+  }
   const R *S0 = sm + L::oS0 + u0 * L::SS, *S1 = sm + L::oS1 + u0 * L::SS;  // the unit's metric buffers
   const Elem<R> x{sm + L::oQ + sh.q + el * L::SQ,
                   sm + L::oBG + sh.bg + el * L::SBG,
@@ -974,10 +978,10 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
   }
   // a refill that gave up (flag set, copies drained): the unit stores none of its elements
   if constexpr (SE) failed |= !mbar_wait(bar + 3, par, A.err, polls);
-  if constexpr (L::SM) {
-    if (warp_local<N>() ? __any_sync(0xffffffffu, failed) : __syncthreads_or(failed)) return;
-  }
+  if constexpr (L::SM) failed = warp_local<N>() ? __any_sync(0xffffffffu, failed) : __syncthreads_or(failed);
   if (!active) return;
+  if (ln == 0) A.skip_out[e] = failed;
+  if (failed) return;
 
   // Thread ln holds its zeta-line's points ln + N^2 i (i < N): consecutive threads read consecutive words
   // of each array.  Inputs that are not staged are loaded one point ahead.
@@ -1150,7 +1154,7 @@ struct UpLayout {
 
 // The end-point fluxes' part of the divergence, added to the volume kernel's output (residual or stage
 // state), and the traces of the new state.  Thread ln holds the points ln + N^2 i of its element.
-// A mesh whose volume kernel gave up a wait (error flag set) is left as it is.  Bound by DRAM: at p = 3,
+// An element for which the volume kernel gave up a wait is left as it is.  Bound by DRAM: at p = 3,
 // 331,776 elements, 5.2 KB an element in 0.307 ms, 84 % of the copy rate.
 template <int N, class R, int EPB, int MODE>
 __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
@@ -1160,7 +1164,7 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
   R* sm = reinterpret_cast<R*>(smem_raw);
   const int el = threadIdx.x / N2, ln = threadIdx.x % N2;
   const int64_t e = tile * EPB + el;
-  const bool active = el < EPB && e < A.m.E;
+  bool active = el < EPB && e < A.m.E;
   R* sF = sm + L::oF + el * L::SF;
   R* sW = sm + L::oW + el * L::SW;
   R W[5][N], ij[N], Fz[2][5];
@@ -1173,7 +1177,7 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
     for (int i = 0; i < N; ++i) ij[i] = __ldg(A.m.invJ + (size_t)e * N3 + ln + N2 * i);
   }
   pdl_wait();
-  const bool flagged = A.err != nullptr && (*(const volatile unsigned*)A.err & 1u) != 0;
+  const int skip = active ? ld_written(A.skip + e) : 1;
   if (active) {
     // the faces' common fluxes at own points, along xi_d: the owner is the lower-numbered element
     R Fxy[20];
@@ -1198,7 +1202,8 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
 #pragma unroll
     for (int c = 0; c < 20; ++c) sF[c * N2 + ln] = Fxy[c];
   }
-  if (__syncthreads_or(flagged)) return;
+  unit_sync<N>();
+  active = skip == 0;
   if (active) {
     const int a = ln % N, b = ln / N;
     const R d0a = A.ops.D[a][0], dNa = A.ops.D[a][N], d0b = A.ops.D[b][0], dNb = A.ops.D[b][N];
@@ -1301,7 +1306,7 @@ struct Launch {
   template <int MODE>
   static cudaError_t vol(const KArgs<R>& A, cudaStream_t st) {
     if (A.m.E == 0) return cudaSuccess;
-    if (A.Tv_out == nullptr || A.T == nullptr) return cudaErrorInvalidValue;
+    if (A.Tv_out == nullptr || A.T == nullptr || A.skip_out == nullptr) return cudaErrorInvalidValue;
     // the radiative-diffusivity profile is a compile-time option of the FP32 kernels (FP64 checks it
     // at run time)
     if constexpr (sizeof(R) == 8) {
@@ -1321,7 +1326,7 @@ struct Launch {
   template <int MODE>
   static cudaError_t update(const KArgs<R>& A, cudaStream_t st) {
     if (A.m.E == 0) return cudaSuccess;
-    if (A.Fc == nullptr || A.out == nullptr) return cudaErrorInvalidValue;
+    if (A.Fc == nullptr || A.out == nullptr || A.skip == nullptr) return cudaErrorInvalidValue;
     const size_t sm = (size_t)UpLayout<N, R, EPB>::total * sizeof(R);
     cudaError_t e = cudaFuncSetAttribute(k_update<N, R, EPB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
