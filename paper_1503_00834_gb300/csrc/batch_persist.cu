@@ -77,7 +77,7 @@ __device__ __noinline__ void trace_item(const PersistArgs& P, int64_t t) {
 }
 template <int S>
 __device__ __noinline__ void vol_item(const PersistArgs& P, int64_t t, uint64_t* bar, uint32_t& pbar) {
-  vol_tile<S + 3, true, float, p_epb<S>(), kModeRK, false>(P.vol[S], t, bar, pbar);
+  vol_tile<S + 3, true, float, p_epb<S>(), false>(P.vol[S], t, bar, pbar);
 }
 template <int S>
 __device__ __noinline__ void face_item(const PersistArgs& P, int64_t t) {
@@ -202,13 +202,13 @@ chorus_status persist_rk3_step(StagePtrs* const groups[4], double dt, unsigned* 
       float* Tn = (k % 2 == 0) ? G.Tb : G.Ta;
       KArgs<float>& a = P.vol[s];
       a.m = G.m; a.ops = G.ops; a.ph = G.ph; a.bg = G.bg; a.q = G.buf[sg.src]; a.T = Tc; a.Tv_out = G.Tv;
-      a.out = G.buf[sg.dst]; a.un = G.buf[sg.un]; a.a = (float)sg.a; a.b = (float)sg.b; a.c = (float)sg.c;
-      a.dt = (float)dt; a.skip_out = G.skip; a.err = err;
+      a.part_out = G.part; a.skip_out = G.skip; a.err = err;
       KArgs<float>& f = P.face[s];
       f.m = G.m; f.ph = G.ph; f.bg = G.bg; f.T = Tc; f.Tv = G.Tv; f.Fc_out = G.Fc; f.err = err;
       KArgs<float>& r = P.update[s];
-      r.m = G.m; r.ops = G.ops; r.Fc = G.Fc; r.out = G.buf[sg.dst]; r.T_out = k + 1 < (int)stg.size() ? Tn : nullptr;
-      r.c = (float)sg.c;
+      r.m = G.m; r.ops = G.ops; r.Fc = G.Fc; r.part = G.part; r.q = G.buf[sg.src]; r.out = G.buf[sg.dst];
+      r.T_out = k + 1 < (int)stg.size() ? Tn : nullptr;
+      r.un = G.buf[sg.un]; r.a = (float)sg.a; r.b = (float)sg.b; r.c = (float)sg.c;
       r.dt = (float)dt; r.skip = G.skip;
       P.faces[s] = G.faces;
       P.nf[s] = G.nf;

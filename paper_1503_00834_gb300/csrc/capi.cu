@@ -470,7 +470,8 @@ size_t ws_words(const chorus_mesh_s* m) {
   const size_t N = m->N, E = m->E;
   const size_t N2 = N * N, N3 = N2 * N;
   // stage buffer + two trace buffers + one-sided viscous face fluxes + two more stage buffers (RK(5,4))
-  // + the gradient record of the three-pass kernels + the common face fluxes of every face point
+  // + the gradient record of the three-pass kernels, where the other stages keep the partial residual and
+  // the marks of the elements to skip + the common face fluxes of every face point
   return 3 * E * 5 * N3 + 2 * E * 6 * 5 * N2 + E * 6 * 4 * N2 + E * 12 * N3 + E * 6 * 5 * N2;
 }
 
@@ -484,7 +485,8 @@ struct Ws {
   R* B;
   R* G;
   R* Fc;
-  int* skip;  // [E] in G, which the stage kernels that use the marks leave alone
+  R* part;    // [E][5][N^3] in G
+  int* skip;  // [E] in G, after part
 };
 
 template <class R>
@@ -501,7 +503,8 @@ Ws<R> split_ws(const chorus_mesh_s* m, void* w) {
   r.B = r.A + E * 5 * N3;
   r.G = r.B + E * 5 * N3;
   r.Fc = r.G + E * 12 * N3;
-  r.skip = (int*)r.G;
+  r.part = r.G;
+  r.skip = (int*)(r.part + E * 5 * N3);
   return r;
 }
 
@@ -902,12 +905,12 @@ chorus_status chorus_residual(chorus_mesh m, const chorus_params* P, chorus_prec
     }
     CHK(timed(m, 0, st, [&] { return m->L.trace64(ma, m->ops64, (const double*)Q, w.Ta, st); }));
     CHK(timed(m, 1, st, [&] {
-      return m->L.vol64(ma, m->ops64, ph, (const double*)Q, w.Ta, w.Tv, (double*)R, rc, 0.0, kModeResidual,
-                         w.skip, m->d_err, st);
+      return m->L.vol64(ma, m->ops64, ph, (const double*)Q, w.Ta, w.Tv, (double*)R, rc.radd, w.skip, m->d_err, st);
     }));
     CHK(timed(m, 3, st, [&] { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
     CHK(timed(m, 2, st, [&] {
-      return m->L.update64(ma, m->ops64, w.Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, w.skip, st);
+      return m->L.update64(ma, m->ops64, nullptr, (const double*)R, w.Fc, (double*)R, nullptr, rc, 0.0, kModeResidual,
+                           w.skip, st);
     }));
     return CHORUS_OK;
   }
@@ -926,12 +929,12 @@ chorus_status chorus_residual(chorus_mesh m, const chorus_params* P, chorus_prec
   }
   CHK(timed(m, 0, st, [&] { return m->L.trace32(ma, m->ops32, (const float*)Q, w.Ta, st); }));
   CHK(timed(m, 1, st, [&] {
-    return m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, (float*)R, rc, 0.0f, kModeResidual,
-                       w.skip, m->d_err, st);
+    return m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, (float*)R, rc.radd, w.skip, m->d_err, st);
   }));
   CHK(timed(m, 3, st, [&] { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
   CHK(timed(m, 2, st, [&] {
-    return m->L.update32(ma, m->ops32, w.Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, w.skip, st);
+    return m->L.update32(ma, m->ops32, nullptr, (const float*)R, w.Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual,
+                         w.skip, st);
   }));
   return CHORUS_OK;
 }
@@ -978,11 +981,11 @@ chorus_status run_rk(chorus_mesh_s* m, R* u, const Ws<R>& w, double dt, int64_t 
                             m->closure_buf, m->E, 0, m->d_err, st));
         c.radd = (const R*)m->closure_buf;
       }
-      CHK(timed(m, 1, st, [&] { return vol(buf[g.src], Tc, buf[g.dst], c); }));
+      CHK(timed(m, 1, st, [&] { return vol(buf[g.src], Tc, c.radd); }));
       CHK(timed(m, 3, st, [&] { return face(Tc); }));
       // the traces of the call's last state are read by nobody: the next call starts with its own
       R* T_out = n + 1 == n_steps && &g == &stg.back() ? nullptr : Tn;
-      CHK(timed(m, 2, st, [&] { return update(buf[g.dst], T_out, c); }));
+      CHK(timed(m, 2, st, [&] { return update(buf[g.src], buf[g.dst], T_out, c); }));
       std::swap(Tc, Tn);
     }
   return CHORUS_OK;
@@ -1038,22 +1041,24 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
   bool copied = false;  // the chunks of the last stage copied the state out
   const chorus_status s = run_rk<float>(
       m, Qd, w, dt, n_steps, 0, st,
-      [&](const float* q, const float* T, float* dst, const RkCoef<float>& c) {
-        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, dst, c, (float)dt, kModeRK, w.skip, m->d_err, st);
+      [&](const float* q, const float* T, const float* radd) {
+        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, w.part, radd, w.skip, m->d_err, st);
       },
       [&](const float* T) { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
-      [&](float* dst, float* Tn, const RkCoef<float>& c) -> cudaError_t {
+      [&](const float* q, float* dst, float* Tn, const RkCoef<float>& c) -> cudaError_t {
         if (++stage < last || dst != Qd)
-          return m->L.update32(ma, m->ops32, w.Fc, dst, Tn, c, (float)dt, kModeRK, w.skip, st);
+          return m->L.update32(ma, m->ops32, q, w.part, w.Fc, dst, Tn, c, (float)dt, kModeRK, w.skip, st);
         for (int k = 0; k < kHostChunks; ++k) {
           int64_t e0, ne;
           range(k, &e0, &ne);
           if (ne == 0) continue;
           RkCoef<float> ck = c;
           const int64_t o5 = e0 * 5 * N3;
+          ck.un = c.un ? c.un + o5 : nullptr;
+          ck.un2 = c.un2 ? c.un2 + o5 : nullptr;
           ck.out2 = c.out2 ? c.out2 + o5 : nullptr;
-          cudaError_t e = m->L.update32(mesh_range(ma, e0, ne, N), m->ops32, w.Fc, dst + o5, Tn, ck, (float)dt, kModeRK,
-                                          w.skip + e0, st);
+          cudaError_t e = m->L.update32(mesh_range(ma, e0, ne, N), m->ops32, q + o5, w.part + o5, w.Fc, dst + o5, Tn, ck,
+                                        (float)dt, kModeRK, w.skip + e0, st);
           if (e == cudaSuccess) e = cudaEventRecord(m->copy_ev[k], st);
           if (e == cudaSuccess) e = cudaStreamWaitEvent(m->copy_stream, m->copy_ev[k], 0);
           if (e == cudaSuccess)
@@ -1146,12 +1151,12 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
     Ws<double> w = split_ws<double>(m, workspace);
     return run_rk<double>(
         m, (double*)Q, w, dt, n_steps, scheme, st,
-        [&](const double* q, const double* T, double* dst, const RkCoef<double>& c) {
-          return m->L.vol64(ma, m->ops64, ph, q, T, w.Tv, dst, c, dt, kModeRK, w.skip, m->d_err, st);
+        [&](const double* q, const double* T, const double* radd) {
+          return m->L.vol64(ma, m->ops64, ph, q, T, w.Tv, w.part, radd, w.skip, m->d_err, st);
         },
         [&](const double* T) { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
-        [&](double* dst, double* Tn, const RkCoef<double>& c) {
-          return m->L.update64(ma, m->ops64, w.Fc, dst, Tn, c, dt, kModeRK, w.skip, st);
+        [&](const double* q, double* dst, double* Tn, const RkCoef<double>& c) {
+          return m->L.update64(ma, m->ops64, q, w.part, w.Fc, dst, Tn, c, dt, kModeRK, w.skip, st);
         },
         [&](const double* q, double* T) { return m->L.trace64(ma, m->ops64, q, T, st); });
   }
@@ -1166,29 +1171,27 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
   if (scheme == 1) {  // on the three-pass kernels (three_pass.cuh)
     ma.x = m->d_x32;
     bg.bgT = m->d_bgTo;
-    const float* src = nullptr;
     return run_rk<float>(
         m, (float*)Q, w, dt, n_steps, scheme, st,
-        [&](const float* q, const float* T, float*, const RkCoef<float>&) {
-          src = q;
+        [&](const float* q, const float* T, const float*) {
           return m->L3.grad(ma, m->ops32, ph, bg, q, T, w.Tv, w.G, m->d_err, st);
         },
         [&](const float* T) {
           return m->L3.face(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st);
         },
-        [&](float* dst, float* Tn, const RkCoef<float>& c) {
-          return m->L3.resid(ma, m->ops32, ph, bg, src, w.G, w.Fc, dst, Tn, c, (float)dt, m->d_err, st);
+        [&](const float* q, float* dst, float* Tn, const RkCoef<float>& c) {
+          return m->L3.resid(ma, m->ops32, ph, bg, q, w.G, w.Fc, dst, Tn, c, (float)dt, m->d_err, st);
         },
         [&](const float* q, float* T) { return m->L3.trace(ma, m->ops32, q, T, st); });
   }
   return run_rk<float>(
       m, (float*)Q, w, dt, n_steps, scheme, st,
-      [&](const float* q, const float* T, float* dst, const RkCoef<float>& c) {
-        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, dst, c, (float)dt, kModeRK, w.skip, m->d_err, st);
+      [&](const float* q, const float* T, const float* radd) {
+        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, w.part, radd, w.skip, m->d_err, st);
       },
       [&](const float* T) { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
-      [&](float* dst, float* Tn, const RkCoef<float>& c) {
-        return m->L.update32(ma, m->ops32, w.Fc, dst, Tn, c, (float)dt, kModeRK, w.skip, st);
+      [&](const float* q, float* dst, float* Tn, const RkCoef<float>& c) {
+        return m->L.update32(ma, m->ops32, q, w.part, w.Fc, dst, Tn, c, (float)dt, kModeRK, w.skip, st);
       },
       [&](const float* q, float* T) { return m->L.trace32(ma, m->ops32, q, T, st); });
 }
@@ -1595,9 +1598,10 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
       rc.radd = (const double*)m->closure_buf;
     }
     CHK(m->L.trace64(ma, m->ops64, (const double*)Q, T, st));
-    CHK(m->L.vol64(ma, m->ops64, ph, (const double*)Q, T, Tv, (double*)R, rc, 0.0, kModeResidual, skip, m->d_err, st));
+    CHK(m->L.vol64(ma, m->ops64, ph, (const double*)Q, T, Tv, (double*)R, rc.radd, skip, m->d_err, st));
     CHK(m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st));
-    CHK(m->L.update64(ma, m->ops64, Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, skip, st));
+    CHK(m->L.update64(ma, m->ops64, nullptr, (const double*)R, Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, skip,
+                      st));
     return CHORUS_OK;
   }
   const PhysArg<float> ph = phys_arg<float>(*P, m->r_inner, m->r_outer);
@@ -1613,9 +1617,9 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
     rc.radd = (const float*)m->closure_buf;
   }
   CHK(m->L.trace32(ma, m->ops32, (const float*)Q, T, st));
-  CHK(m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, (float*)R, rc, 0.0f, kModeResidual, skip, m->d_err, st));
+  CHK(m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, (float*)R, rc.radd, skip, m->d_err, st));
   CHK(m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st));
-  CHK(m->L.update32(ma, m->ops32, Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, skip, st));
+  CHK(m->L.update32(ma, m->ops32, nullptr, (const float*)R, Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, skip, st));
   return CHORUS_OK;
 }
 
@@ -1679,6 +1683,7 @@ chorus_status mesh_stage_ptrs(chorus_mesh_s* m, const chorus_params& P, float* u
   out->Tb = w.Tb;
   out->Tv = w.Tv;
   out->Fc = w.Fc;
+  out->part = w.part;
   out->skip = w.skip;
   out->faces = m->d_faces;
   out->nf = m->n_ifaces;

@@ -69,7 +69,7 @@ __host__ __device__ inline int bg_point(int N, int pt) {
 
 enum ResidMode { kModeResidual = 0, kModeRK = 1 };
 
-// Stage combination of the RK update fused into the volume kernel:
+// Stage combination of the RK update fused into the update kernel:
 //   out  = a un  + b q + c dt R
 //   out2 = a2 un2 + b2 q + c2 dt R   (when out2 != nullptr)
 // where R includes `radd` (an additive residual correction, e.g. the learned closure) when non-null.
@@ -85,31 +85,34 @@ struct RkCoef {
 
 // Per-order launchers (defined in kern_p<N>.cu).  All return cudaGetLastError().
 //   trace   face traces of q, each in the neighbour's slot (trace_slot); T: of the whole mesh
-//   vol     from q and its traces: one-sided viscous face fluxes Tv and `out`, the residual (mode
-//           kModeResidual) or stage state (kModeRK, and rk.out2) without the end-point fluxes; `out` may be q
+//   vol     from q and its traces: one-sided viscous face fluxes Tv and `part`, the residual without the
+//           end-point fluxes; radd: an additive residual correction (e.g. the learned closure) or null
 //   face    common fluxes Fc [faces][5][N^2], along the owner's outward S, of the face list (n_faces
 //           interior faces, from their lower element, then n_walls wall faces)
-//   update  the end-point fluxes' part added to `out` (and rk.out2); T_out: traces of the new state
-//           (of the whole mesh)
+//   update  `out` from `part` and the end-point fluxes: the residual (mode kModeResidual; `out` may be
+//           `part`) or the stage state (kModeRK, and rk.out2; `out` may be q or rk.un), with T_out its
+//           traces (of the whole mesh)
 // skip [E]: vol marks the elements whose staging gave up (it stores nothing for them), update leaves
 // those as they are.
 struct LaunchSet {
   cudaError_t (*trace64)(const MeshArg<double>&, const OpsArg<double>&, const double* q, double* T, cudaStream_t);
   cudaError_t (*vol64)(const MeshArg<double>&, const OpsArg<double>&, const PhysArg<double>&, const double* q,
-                       const double* T, double* Tv, double* out, const RkCoef<double>& rk,
-                       double dt, int mode, int* skip, unsigned* err, cudaStream_t);
+                       const double* T, double* Tv, double* part, const double* radd, int* skip, unsigned* err,
+                       cudaStream_t);
   cudaError_t (*face64)(const MeshArg<double>&, const PhysArg<double>&, const int2* faces, int n_faces, int n_walls,
                         const double* T, const double* Tv, double* Fc, cudaStream_t);
-  cudaError_t (*update64)(const MeshArg<double>&, const OpsArg<double>&, const double* Fc, double* out, double* T_out,
-                          const RkCoef<double>& rk, double dt, int mode, const int* skip, cudaStream_t);
+  cudaError_t (*update64)(const MeshArg<double>&, const OpsArg<double>&, const double* q, const double* part,
+                          const double* Fc, double* out, double* T_out, const RkCoef<double>& rk, double dt, int mode,
+                          const int* skip, cudaStream_t);
   cudaError_t (*trace32)(const MeshArg<float>&, const OpsArg<float>&, const float* q, float* T, cudaStream_t);
   cudaError_t (*vol32)(const MeshArg<float>&, const OpsArg<float>&, const PhysArg<float>&, const BgArg&,
-                       const float* q, const float* T, float* Tv, float* out, const RkCoef<float>& rk, float dt,
-                       int mode, int* skip, unsigned* err, cudaStream_t);
+                       const float* q, const float* T, float* Tv, float* part, const float* radd, int* skip,
+                       unsigned* err, cudaStream_t);
   cudaError_t (*face32)(const MeshArg<float>&, const PhysArg<float>&, const BgArg&, const int2* faces, int n_faces,
                         int n_walls, const float* T, const float* Tv, float* Fc, cudaStream_t);
-  cudaError_t (*update32)(const MeshArg<float>&, const OpsArg<float>&, const float* Fc, float* out, float* T_out,
-                          const RkCoef<float>& rk, float dt, int mode, const int* skip, cudaStream_t);
+  cudaError_t (*update32)(const MeshArg<float>&, const OpsArg<float>&, const float* q, const float* part,
+                          const float* Fc, float* out, float* T_out, const RkCoef<float>& rk, float dt, int mode,
+                          const int* skip, cudaStream_t);
   int epb32;  // elements per CTA of the FP32 volume kernel
 };
 

@@ -13,30 +13,21 @@ struct Inst {
   static cudaError_t trace(const MeshArg<R>& m, const OpsArg<R>& ops, const R* q, R* T, cudaStream_t st) {
     return Launch<N, PERT, R, EPB>::trace(m, ops, q, T, st);
   }
-  template <class R>
-  static void set_rk(KArgs<R>& A, const RkCoef<R>& rk) {
-    A.un = rk.un; A.a = rk.a; A.b = rk.b; A.c = rk.c;
-    A.un2 = rk.un2; A.out2 = rk.out2; A.a2 = rk.a2; A.b2 = rk.b2; A.c2 = rk.c2; A.radd = rk.radd;
-  }
   static cudaError_t vol64(const MeshArg<double>& m, const OpsArg<double>& ops, const PhysArg<double>& ph,
-                           const double* q, const double* T, double* Tv, double* out,
-                           const RkCoef<double>& rk, double dt, int mode, int* skip, unsigned* err, cudaStream_t st) {
-    using L = Launch<N, false, double, EPB64>;
+                           const double* q, const double* T, double* Tv, double* part, const double* radd, int* skip,
+                           unsigned* err, cudaStream_t st) {
     KArgs<double> A{};
-    A.m = m; A.ops = ops; A.ph = ph; A.q = q; A.T = T; A.Tv_out = Tv; A.out = out;
-    set_rk(A, rk);
-    A.dt = dt; A.skip_out = skip; A.err = err;
-    return mode == kModeRK ? L::template vol<kModeRK>(A, st) : L::template vol<kModeResidual>(A, st);
+    A.m = m; A.ops = ops; A.ph = ph; A.q = q; A.T = T; A.Tv_out = Tv; A.part_out = part; A.radd = radd;
+    A.skip_out = skip; A.err = err;
+    return Launch<N, false, double, EPB64>::vol(A, st);
   }
   static cudaError_t vol32(const MeshArg<float>& m, const OpsArg<float>& ops, const PhysArg<float>& ph,
-                           const BgArg& bg, const float* q, const float* T, float* Tv, float* out,
-                           const RkCoef<float>& rk, float dt, int mode, int* skip, unsigned* err, cudaStream_t st) {
-    using L = Launch<N, true, float, EPB32>;
+                           const BgArg& bg, const float* q, const float* T, float* Tv, float* part, const float* radd,
+                           int* skip, unsigned* err, cudaStream_t st) {
     KArgs<float> A{};
-    A.m = m; A.ops = ops; A.ph = ph; A.bg = bg; A.q = q; A.T = T; A.Tv_out = Tv; A.out = out;
-    set_rk(A, rk);
-    A.dt = dt; A.skip_out = skip; A.err = err;
-    return mode == kModeRK ? L::template vol<kModeRK>(A, st) : L::template vol<kModeResidual>(A, st);
+    A.m = m; A.ops = ops; A.ph = ph; A.bg = bg; A.q = q; A.T = T; A.Tv_out = Tv; A.part_out = part; A.radd = radd;
+    A.skip_out = skip; A.err = err;
+    return Launch<N, true, float, EPB32>::vol(A, st);
   }
   static cudaError_t face64(const MeshArg<double>& m, const PhysArg<double>& ph, const int2* faces, int nf, int nw,
                             const double* T, const double* Tv, double* Fc, cudaStream_t st) {
@@ -51,12 +42,13 @@ struct Inst {
     return Launch<N, true, float, EPB32>::face(A, faces, nf, nw, st);
   }
   template <bool PERT, class R, int EPB>
-  static cudaError_t update(const MeshArg<R>& m, const OpsArg<R>& ops, const R* Fc, R* out, R* T_out,
-                            const RkCoef<R>& rk, R dt, int mode, const int* skip, cudaStream_t st) {
+  static cudaError_t update(const MeshArg<R>& m, const OpsArg<R>& ops, const R* q, const R* part, const R* Fc, R* out,
+                            R* T_out, const RkCoef<R>& rk, R dt, int mode, const int* skip, cudaStream_t st) {
     using L = Launch<N, PERT, R, EPB>;
     KArgs<R> A{};
-    A.m = m; A.ops = ops; A.Fc = Fc; A.out = out; A.T_out = T_out;
-    set_rk(A, rk);
+    A.m = m; A.ops = ops; A.q = q; A.part = part; A.Fc = Fc; A.out = out; A.T_out = T_out;
+    A.un = rk.un; A.a = rk.a; A.b = rk.b; A.c = rk.c;
+    A.un2 = rk.un2; A.out2 = rk.out2; A.a2 = rk.a2; A.b2 = rk.b2; A.c2 = rk.c2;
     A.dt = dt; A.skip = skip;
     return mode == kModeRK ? L::template update<kModeRK>(A, st) : L::template update<kModeResidual>(A, st);
   }

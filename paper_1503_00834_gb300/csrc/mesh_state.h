@@ -108,7 +108,7 @@ struct StagePtrs {
   PhysArg<float> ph;
   BgArg bg;
   float* buf[4];  // stage buffers: u, s, A, B (ids of Stage)
-  float *Ta, *Tb, *Tv, *Fc;
+  float *Ta, *Tb, *Tv, *part, *Fc;
   int* skip;
   const int2* faces;
   int nf, nw;

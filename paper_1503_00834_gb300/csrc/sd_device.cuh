@@ -108,6 +108,10 @@ __device__ __forceinline__ bool mbar_wait0(uint64_t* bar, unsigned* err, uint32_
   return mbar_wait(bar, 0u, err, polls);
 }
 
+// One rounding, in the operands' own type.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // ------------------------------------------------------------------ index helpers
 
 // point index of position s along line `ln` of direction d

@@ -3,12 +3,16 @@
 // A residual (and an RK stage) is three kernels:
 //   k_vol     everything an element can do alone once its neighbours' traces are known: the lifted
 //             gradients, the one-sided viscous flux of every face point (written for both sides), the
-//             fluxes at the interior flux points, their part of the divergence, the sources and the
-//             RK combination.  Writes the new state without the two end-point fluxes of each line.
+//             fluxes at the interior flux points, their part of the divergence and the sources.
+//             Writes the residual without the two end-point fluxes of each line.
 //   k_face    the common flux of every face point, once per face, from both sides' traces.
-//   k_update  adds the end-point fluxes' part of the divergence and writes the new state's traces.
-// The gradient record never leaves the SM, and the state, the metrics and the background are read
-// once a stage.
+//   k_update  adds the end-point fluxes' part of the divergence, forms the RK combination and writes the
+//             new state's traces.
+// The gradient record never leaves the SM, and the metrics and the background are read once a stage.
+// The state is read again by k_update, so that the new state is rounded once, from the whole residual:
+// with the combination in k_vol and the end-point fluxes added to its rounded result (one read of the state
+// less; p = 3, 331,776 elements: 1.82 against 1.88 ms a stage) a step was 7 to 17 % further from the 64-bit
+// one, at every order.
 //
 // k_vol: one CTA processes EPB elements; each element is handled by N*N threads, thread `ln` owning
 // the line (a, b) = (ln % N, ln / N) of every direction (xi-line (j,k), eta-line (i,k), zeta-line
@@ -86,7 +90,7 @@ __host__ __device__ constexpr int unit_threads() { return warp_local<N>() ? 32 :
 template <int N, class R>
 __host__ __device__ constexpr bool stage_metrics() { return sizeof(R) == 4 && N <= 4; }
 
-// Whether the epilogue's inputs (R(Q0), u^n, x) are staged too, by bulk copies into the record's and a
+// Whether the epilogue's inputs (R(Q0), x) are staged too, by bulk copies into the record's and a
 // metric buffer's space once the last sweep has its lines in registers, so that they arrive during
 // that sweep: left to register loads after it, they were the longest stall of the kernel (0.41 of
 // 1.79 ms at p = 3, 331,776 elements).
@@ -133,18 +137,20 @@ struct KArgs {
   OpsArg<R> ops;
   PhysArg<R> ph;
   BgArg bg;            // perturbation form only
-  const R* q;          // state (form variables)
+  const R* q;          // state (form variables); k_update: in RK mode
   const R* T;          // face traces of q, [E][6][5][N2] (trace_slot)
   const R* Tv;         // one-sided viscous fluxes along the outward S [E][6][4][N2] (k_face input)
   R* Tv_out;           // k_vol output
-  R* out;              // residual or new state (k_vol: without the end-point fluxes; k_update: completed)
+  R* part_out;         // k_vol output: the residual without the end-point fluxes [E][5][N3]
+  const R* part;       // k_update input
+  R* out;              // k_update: residual or new state
   R* T_out;            // k_update: traces of the new state (RK mode)
   const R* un;         // first extra state of the RK combination
   R a, b, c, dt;       // out = a un + b q + c dt R
   const R* un2;        // optional second output: out2 = a2 un2 + b2 q + c2 dt R
   R* out2;
   R a2, b2, c2;
-  const R* radd;       // optional additive residual correction [E][5][N3]
+  const R* radd;       // k_vol: optional additive residual correction [E][5][N3]
   R* Fc_out;           // k_face output: common fluxes along the owner's outward S [faces][5][N2]
   const R* Fc;         // k_update input
   int* skip_out;       // k_vol: per element, 1 if its staging gave up (nothing stored for it), else 0
@@ -845,10 +851,10 @@ __device__ __forceinline__ void add_div(const Elem<R>& x, int ln, const R (&acc)
 // ------------------------------------------------------------------ volume kernel
 
 // Bound by instruction issue and the latency of dependent instructions at the warps that registers
-// allow: at p = 3 in FP32 (331,776 elements) 1.19 ms for 13.6 KB of DRAM traffic an element, 58 % of the
+// allow: at p = 3 in FP32 (331,776 elements) 1.15 ms for 13.6 KB of DRAM traffic an element, 58 % of the
 // issue slots at 12 warps per SM, DRAM at 46 %; the lifting and residual kernels that it replaces took 1.97 ms,
-// 28.9 KB and 1.4 times the instructions.  p = 2 (98,304 elements) 0.52 -> 0.19 ms, p = 4 (111,078) 2.92 ->
-// 1.00 ms (shared-memory pipe 62 %), p = 5 (98,304) 3.34 -> 1.88 ms; FP64 at p = 3 43.7 -> 32.7 ms, at the
+// 28.9 KB and 1.4 times the instructions.  p = 2 (98,304 elements) 0.52 -> 0.18 ms, p = 4 (111,078) 2.92 ->
+// 0.97 ms (shared-memory pipe 62 %), p = 5 (98,304) 3.34 -> 1.85 ms; FP64 at p = 3 43.7 -> 31.9 ms, at the
 // FP64 units' rate.
 
 // Barriers of a unit: the staging, the two refills of the metric buffers, and the epilogue's inputs.
@@ -856,7 +862,7 @@ constexpr int kVolBars = 4;
 
 // Tile `tile` (elements tile * EPB ...; threads beyond EPB * N^2 idle but take part in the barriers).
 // bars: the CTA's barriers, kVolBars for each unit (initialised), pbar: the parity of their next phase.
-template <int N, bool PERT, class R, int EPB, int MODE, bool KR>
+template <int N, bool PERT, class R, int EPB, bool KR>
 __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64_t* bars, uint32_t& pbar) {
   using L = Layout<N, PERT, R, EPB>;
   constexpr int N2 = N * N, N3 = N * N * N;
@@ -943,17 +949,14 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
   }
   if constexpr (L::SM) failed |= !mbar_wait(bar + 2, par, A.err, polls);
   unit_sync<N>();
-  // the epilogue's inputs: staged (SE) into the record's space (R(Q0), then u^n) and the free metric
-  // buffer (x), a stage whose combination has no u^n term (a = 0) not reading it
+  // the epilogue's inputs: staged (SE) into the record's space (R(Q0)) and the free metric buffer (x)
   constexpr bool SE = PERT && stage_epilogue<N, R>();
-  const bool want_un = MODE == kModeRK && A.a != R(0), want_r0 = PERT && A.bg.R0 != nullptr;
-  const bool bulk_un = SE && want_un && ((uintptr_t)A.un & 15u) == 0;
+  const bool want_r0 = PERT && A.bg.R0 != nullptr;
   const unsigned lanes = SE ? __ballot_sync(0xffffffffu, active) : 0u;
   if constexpr (PERT && !SE) {
     if (tid == 0) {
       prefetch_l2(A.m.x + (size_t)e0 * 3 * N3, ne * 3 * N3 * sizeof(R));
       if (want_r0) prefetch_l2(A.bg.R0 + (size_t)e0 * 5 * N3, ne * 5 * N3 * sizeof(R));
-      if (want_un) prefetch_l2(A.un + (size_t)e0 * 5 * N3, ne * 5 * N3 * sizeof(R));
     }
   }
   auto stage_late = [&] {
@@ -962,11 +965,9 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
       if (tid == 0) {
         fence_async_smem();
         constexpr uint32_t b5 = 5 * N3 * sizeof(R), b3 = 3 * N3 * sizeof(R);
-        mbar_expect_tx(bar + 3, ne * ((want_r0 ? b5 : 0) + (bulk_un ? b5 : 0) + b3));
+        mbar_expect_tx(bar + 3, ne * ((want_r0 ? b5 : 0) + b3));
         for (int j = 0; j < ne; ++j) {
-          R* g = sm + L::oG + (u0 + j) * L::SG;
-          if (want_r0) bulk_g2s(g, A.bg.R0 + (size_t)(e0 + j) * 5 * N3, b5, bar + 3);
-          if (bulk_un) bulk_g2s(g + 5 * N3, A.un + (size_t)(e0 + j) * 5 * N3, b5, bar + 3);
+          if (want_r0) bulk_g2s(sm + L::oG + (u0 + j) * L::SG, A.bg.R0 + (size_t)(e0 + j) * 5 * N3, b5, bar + 3);
           bulk_g2s(const_cast<R*>(S0) + j * L::SS, A.m.x + (size_t)(e0 + j) * 3 * N3, b3, bar + 3);
         }
       }
@@ -986,7 +987,7 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
   // Thread ln holds its zeta-line's points ln + N^2 i (i < N): consecutive threads read consecutive words
   // of each array.  Inputs that are not staged are loaded one point ahead.
   struct In {
-    R x[3], ij, r0[5], un[5];
+    R x[3], ij, r0[5];
   };
   auto load_in = [&](int i) {
     In v;
@@ -996,21 +997,14 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
     v.ij = L::SM ? x.ij[pt] : __ldg(A.m.invJ + (size_t)e * N3 + pt);
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
-      const size_t oi = ((size_t)e * 5 + c) * N3 + pt;
-      if constexpr (SE) {
-        v.r0[c] = want_r0 ? x.g[c * N3 + pt] : R(0);
-        v.un[c] = bulk_un ? x.g[(5 + c) * N3 + pt] : want_un ? A.un[oi] : R(0);
-      } else {
-        v.r0[c] = want_r0 ? (R)__ldg(A.bg.R0 + oi) : R(0);
-        v.un[c] = want_un ? A.un[oi] : R(0);
-      }
+      if constexpr (SE) v.r0[c] = want_r0 ? x.g[c * N3 + pt] : R(0);
+      else v.r0[c] = want_r0 ? (R)__ldg(A.bg.R0 + ((size_t)e * 5 + c) * N3 + pt) : R(0);
     }
     return v;
   };
-  // residual dQ/dt = -div/|J| - M (Eqs. 4, 11) without the end points, sources of Eqs. 2-3, and the RK
-  // combination
+  // residual dQ/dt = -div/|J| - M (Eqs. 4, 11) without the end points, sources of Eqs. 2-3
   const PhysArg<R>& ph = A.ph;
-  auto finish = [&](auto extra) {  // extra: an additive correction or a second output
+  auto finish = [&](auto extra) {  // extra: an additive correction
     In cur, nxt = load_in(0);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -1038,22 +1032,16 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
         R Rv = -(x.g[(kG + v) * N3 + si] + acc[v][i]) * cur.ij - M[v];
         if (PERT) Rv += cur.r0[v];
         const size_t oi = ((size_t)e * 5 + v) * N3 + pt;
-        if (decltype(extra)::value && A.radd) Rv += ld_written(A.radd + oi);
-        if (MODE == kModeResidual) {
-          A.out[oi] = Rv;
-        } else {
-          const R dR = A.dt * Rv;
-          if (decltype(extra)::value && A.out2) A.out2[oi] = A.a2 * A.un2[oi] + A.b2 * q[v] + A.c2 * dR;
-          A.out[oi] = A.a * cur.un[v] + A.b * q[v] + A.c * dR;
-        }
+        if (decltype(extra)::value) Rv += ld_written(A.radd + oi);
+        A.part_out[oi] = Rv;
       }
     }
   };
-  if (A.radd != nullptr || A.out2 != nullptr) finish(std::true_type{});
+  if (A.radd != nullptr) finish(std::true_type{});
   else finish(std::false_type{});
 }
 
-template <int N, bool PERT, class R, int EPB, int MODE, bool KR>
+template <int N, bool PERT, class R, int EPB, bool KR>
 __global__ void __launch_bounds__(EPB * N * N, sizeof(R) == 4 ? vol_min_blocks<N, EPB>() : 1) k_vol(const KArgs<R> A) {
   constexpr int units = (EPB + unit_elems<N, EPB>() - 1) / unit_elems<N, EPB>();
   __shared__ __align__(8) uint64_t bars[units * kVolBars];
@@ -1061,7 +1049,7 @@ __global__ void __launch_bounds__(EPB * N * N, sizeof(R) == 4 ? vol_min_blocks<N
   if (threadIdx.x < units * kVolBars) mbar_init(&bars[threadIdx.x]);
   __syncthreads();
   uint32_t ph = 0;
-  vol_tile<N, PERT, R, EPB, MODE, KR>(A, blockIdx.x, bars, ph);
+  vol_tile<N, PERT, R, EPB, KR>(A, blockIdx.x, bars, ph);
 }
 
 // ------------------------------------------------------------------ face kernel
@@ -1152,10 +1140,12 @@ struct UpLayout {
   static constexpr int total = oW + EPB * SW;
 };
 
-// The end-point fluxes' part of the divergence, added to the volume kernel's output (residual or stage
-// state), and the traces of the new state.  Thread ln holds the points ln + N^2 i of its element.
-// An element for which the volume kernel gave up a wait is left as it is.  Bound by DRAM: at p = 3,
-// 331,776 elements, 5.2 KB an element in 0.307 ms, 84 % of the copy rate.
+// The end-point fluxes' part of the divergence, added to the volume kernel's partial residual; in RK mode
+// the stage's combination and the traces of the new state.  Thread ln takes the points ln + N^2 i of its
+// element.  An element for which the volume kernel gave up a wait is left as it is.  Bound by DRAM: at p = 3,
+// 331,776 elements, 7.3 KB an element in 0.410 ms, 87 % of the copy rate.  One point's inputs are loaded while the
+// point before is worked on: all of them ahead took 96 registers, which slowed the kernel (0.590 ms) and, no
+// room being left for its early start, a stage of 1,470 elements too (20.4 -> 26.2 us).
 template <int N, class R, int EPB, int MODE>
 __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
   using L = UpLayout<N, R, EPB>;
@@ -1167,17 +1157,35 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
   bool active = el < EPB && e < A.m.E;
   R* sF = sm + L::oF + el * L::SF;
   R* sW = sm + L::oW + el * L::SW;
-  R W[5][N], ij[N], Fz[2][5];
+  constexpr int NI = MODE == kModeRK ? 5 : 1;
+  R Fz[2][5];
   int nbr[6], code[6], fid[6];
   if (active) {
     load_six(A.m.nbr, e, nbr);
     load_six(A.m.code, e, code);
     load_six(A.m.fid, e, fid);
-#pragma unroll
-    for (int i = 0; i < N; ++i) ij[i] = __ldg(A.m.invJ + (size_t)e * N3 + ln + N2 * i);
   }
   pdl_wait();
   const int skip = active ? ld_written(A.skip + e) : 1;
+  // A point's inputs, loaded one point ahead.
+  struct In {
+    R ij, part[5], q[NI], un[NI];
+  };
+  auto load_in = [&](int i) {
+    In in;
+    in.ij = __ldg(A.m.invJ + (size_t)e * N3 + ln + N2 * i);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const size_t oi = ((size_t)e * 5 + v) * N3 + ln + N2 * i;
+      in.part[v] = ld_written(A.part + oi);
+      if constexpr (MODE == kModeRK) {
+        in.q[v] = ld_written(A.q + oi);
+        in.un[v] = A.a != R(0) ? ld_written(A.un + oi) : R(0);  // a stage without a u^n term does not read it
+      }
+    }
+    return in;
+  };
+  In nxt;
   if (active) {
     // the faces' common fluxes at own points, along xi_d: the owner is the lower-numbered element
     R Fxy[20];
@@ -1193,12 +1201,7 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
         else Fz[F < 4 ? 0 : F - 4][v] = f;
       }
     }
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const int pt = ln + N2 * i;
-#pragma unroll
-      for (int v = 0; v < 5; ++v) W[v][i] = A.out[((size_t)e * 5 + v) * N3 + pt];
-    }
+    nxt = load_in(0);
 #pragma unroll
     for (int c = 0; c < 20; ++c) sF[c * N2 + ln] = Fxy[c];
   }
@@ -1207,23 +1210,26 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
   if (active) {
     const int a = ln % N, b = ln / N;
     const R d0a = A.ops.D[a][0], dNa = A.ops.D[a][N], d0b = A.ops.D[b][0], dNb = A.ops.D[b][N];
-    const R cdt = MODE == kModeRK ? A.c * A.dt : R(1);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int pt = ln + N2 * i, si = sidx<N, R>(a, b, i);
+      const In in = nxt;
+      if (i + 1 < N) nxt = load_in(i + 1);
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         R s = A.ops.D[i][0] * Fz[0][v] + A.ops.D[i][N] * Fz[1][v];
         s += d0a * sF[v * N2 + b + N * i] + dNa * sF[(5 + v) * N2 + b + N * i];
         s += d0b * sF[(10 + v) * N2 + a + N * i] + dNb * sF[(15 + v) * N2 + a + N * i];
-        s *= ij[i];
+        s *= in.ij;
         const size_t oi = ((size_t)e * 5 + v) * N3 + pt;
-        W[v][i] -= cdt * s;
-        A.out[oi] = W[v][i];
-        if (MODE == kModeRK) {
-          if (A.out2) A.out2[oi] -= A.c2 * A.dt * s;
-          sW[v * N3 + si] = W[v][i];
+        R w = in.part[v] - s;  // the whole residual
+        if constexpr (MODE == kModeRK) {
+          const R dR = A.dt * w, bq = A.b * in.q[v];
+          if (A.out2) A.out2[oi] = fma_rn(A.c2, dR, fma_rn(A.a2, A.un2[oi], A.b2 * in.q[v]));
+          w = fma_rn(A.c, dR, A.a != R(0) ? fma_rn(A.a, in.un[v], bq) : bq);  // the new state
+          sW[v * N3 + si] = w;
         }
+        A.out[oi] = w;
       }
     }
   }
@@ -1231,6 +1237,8 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
     if (A.T_out == nullptr) return;
     unit_sync<N>();
     if (!active) return;
+    load_six(A.m.nbr, e, nbr);  // again: kept in registers over the points they cost a CTA per SM
+    load_six(A.m.code, e, code);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       R* T0 = A.T_out + trace_slot<N>(A.m.e0 + e, 2 * d, nbr[2 * d], code[2 * d], ln);
@@ -1240,12 +1248,12 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
         R l[N];
         if (d == 0) load_line<N, 0, kComputed>(sW + v * N3, ln, l);
         else if (d == 1) load_line<N, 1, kComputed>(sW + v * N3, ln, l);
+        else load_line<N, 2, kComputed>(sW + v * N3, ln, l);
         R lo = R(0), hi = R(0);
 #pragma unroll
         for (int s = 0; s < N; ++s) {
-          const R val = d == 2 ? W[v][s] : l[s];
-          lo += A.ops.I[0][s] * val;
-          hi += A.ops.I[N][s] * val;
+          lo += A.ops.I[0][s] * l[s];
+          hi += A.ops.I[N][s] * l[s];
         }
         T0[v * N2] = lo;
         T1[v * N2] = hi;
@@ -1303,30 +1311,30 @@ struct Launch {
     // 64-thread CTAs (p = 3: 1 % faster than 128, 2.5 % faster than 256)
     return launch_dependent(early(A.m.E), k_face<N, PERT, R>, (unsigned)((n + 63) / 64), 64, 0, st, A, faces, nf, nw);
   }
-  template <int MODE>
   static cudaError_t vol(const KArgs<R>& A, cudaStream_t st) {
     if (A.m.E == 0) return cudaSuccess;
-    if (A.Tv_out == nullptr || A.T == nullptr || A.skip_out == nullptr) return cudaErrorInvalidValue;
+    if (A.Tv_out == nullptr || A.T == nullptr || A.part_out == nullptr || A.skip_out == nullptr) return cudaErrorInvalidValue;
     // the radiative-diffusivity profile is a compile-time option of the FP32 kernels (FP64 checks it
     // at run time)
     if constexpr (sizeof(R) == 8) {
-      return vol_kr<MODE, true>(A, st);
+      return vol_kr<true>(A, st);
     } else {
-      return A.m.kr != nullptr ? vol_kr<MODE, true>(A, st) : vol_kr<MODE, false>(A, st);
+      return A.m.kr != nullptr ? vol_kr<true>(A, st) : vol_kr<false>(A, st);
     }
   }
-  template <int MODE, bool KR>
+  template <bool KR>
   static cudaError_t vol_kr(const KArgs<R>& A, cudaStream_t st) {
     const size_t sm = (size_t)Layout<N, PERT, R, EPB>::total * sizeof(R);
     cudaError_t e =
-        cudaFuncSetAttribute(k_vol<N, PERT, R, EPB, MODE, KR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(k_vol<N, PERT, R, EPB, KR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    return launch_dependent(early(A.m.E), k_vol<N, PERT, R, EPB, MODE, KR>, blocks(A.m.E), threads, sm, st, A);
+    return launch_dependent(early(A.m.E), k_vol<N, PERT, R, EPB, KR>, blocks(A.m.E), threads, sm, st, A);
   }
   template <int MODE>
   static cudaError_t update(const KArgs<R>& A, cudaStream_t st) {
     if (A.m.E == 0) return cudaSuccess;
-    if (A.Fc == nullptr || A.out == nullptr || A.skip == nullptr) return cudaErrorInvalidValue;
+    if (A.Fc == nullptr || A.part == nullptr || A.out == nullptr || A.skip == nullptr) return cudaErrorInvalidValue;
+    if (MODE == kModeRK && (A.q == nullptr || (A.a != R(0) && A.un == nullptr))) return cudaErrorInvalidValue;
     const size_t sm = (size_t)UpLayout<N, R, EPB>::total * sizeof(R);
     cudaError_t e = cudaFuncSetAttribute(k_update<N, R, EPB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
