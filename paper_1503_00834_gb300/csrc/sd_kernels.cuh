@@ -111,11 +111,12 @@ struct Layout {
   // N = 3 FP32: 443 words, 27 mod 32, so that the xi lines of a warp's elements start in 32 different
   // banks (0.206 -> 0.193 ms at 98,304 elements); no stride measured better at N = 5 and 6
   static constexpr int SG = padded ? pad_stride<R>(16 * N3) : 16 * N3 + (N == 3 && sizeof(R) == 4 ? 11 : 0);
-  // interpolation I[f][s] and derivative D[i][f] as pairs of equal values, indexed by rolled loops
+  // interpolation I[f][s], then derivative D[i][f] as [f][i], as pairs of equal values, indexed by rolled
+  // loops; a table for each unit (only its own threads wait for its stores)
   static constexpr int TAB = 4 * (N + 1) * N;
+  static constexpr int units = (EPB + unit_elems<N, EPB>() - 1) / unit_elems<N, EPB>();
   static constexpr int oI = 0;
-  static constexpr int oD = oI + 2 * (N + 1) * N;  // [f][i]
-  static constexpr int oQ = (oI + TAB + 31) / 32 * 32;
+  static constexpr int oQ = (oI + units * TAB + 31) / 32 * 32;
   static constexpr int oBG = oQ + block(5 * N3);
   static constexpr int oGR0 = oBG + (PERT ? block(2 * N3) : 0);
   static constexpr int oG = oGR0 + (PERT ? block(3 * N3) : 0);
@@ -881,15 +882,16 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
   if (ne == 0) return;  // the same in every thread of the unit
   const uint32_t polls = wait_polls(A.err);
   const uint32_t par = pbar;
+  R* tab = sm + L::oI + unit * L::TAB;
   LiftPre<N, R, L::SM> pre[L::SM ? 3 : 1];
   int nbr[6] = {0, 0, 0, 0, 0, 0};
   if (active) load_six(A.m.nbr, e, nbr);
   Shift sh;
   if (!stage_elements<N, PERT, R, EPB>(A, sm, bar, pbar, e0, ne, u0, tid, UT, sh, polls, [&] {
-        // operator tables, each value as a pair; every unit writes the same values
+        // operator tables, each value as a pair
         for (int i = tid; i < 2 * (N + 1) * N; i += UT) {
           const R w = __ldg(A.m.tab + i);
-          *reinterpret_cast<Pair<R>*>(sm + L::oI + 2 * i) = Pair<R>{w, w};
+          *reinterpret_cast<Pair<R>*>(tab + 2 * i) = Pair<R>{w, w};
         }
         if (!active) return;
         lift_prefetch<N, R, 2, L::SM>(A, e, ln, pre[0], nbr);
@@ -933,7 +935,6 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
   unit_sync<N>();
   if (active) lift_dir<N, PERT, R, 0, L::SM>(A, x, ln, e, pre[L::SM ? 2 : 0]);
   unit_sync<N>();
-  const R* tab = sm + L::oI;
   R acc[5][N];
   if (active) {
     const int kind[2] = {nbr[2], nbr[3]};
@@ -1043,7 +1044,7 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
 
 template <int N, bool PERT, class R, int EPB, bool KR>
 __global__ void __launch_bounds__(EPB * N * N, sizeof(R) == 4 ? vol_min_blocks<N, EPB>() : 1) k_vol(const KArgs<R> A) {
-  constexpr int units = (EPB + unit_elems<N, EPB>() - 1) / unit_elems<N, EPB>();
+  constexpr int units = Layout<N, PERT, R, EPB>::units;
   __shared__ __align__(8) uint64_t bars[units * kVolBars];
   pdl_trigger();
   if (threadIdx.x < units * kVolBars) mbar_init(&bars[threadIdx.x]);
