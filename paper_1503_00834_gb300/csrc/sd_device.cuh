@@ -85,7 +85,6 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity, uint32_
   }
   return false;
 }
-__device__ __forceinline__ bool mbar_try0(uint64_t* bar, uint32_t polls) { return mbar_try(bar, 0u, polls); }
 
 // The device control block of a mesh: err[0] error flags, err[1] the wait limit (0: the default,
 // k + 1: k polls).  Returns the number of polls of a kernel's staging waits.
@@ -104,24 +103,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsign
   mbar_try(bar, parity, kDefaultWaitPolls);
   return false;
 }
-__device__ __forceinline__ bool mbar_wait0(uint64_t* bar, unsigned* err, uint32_t polls) {
-  return mbar_wait(bar, 0u, err, polls);
-}
 
 // One rounding, in the operands' own type.
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // ------------------------------------------------------------------ index helpers
-
-// point index of position s along line `ln` of direction d
-template <int N>
-__device__ __forceinline__ int pt_of(int d, int ln, int s) {
-  const int t1 = ln % N, t2 = ln / N;
-  if (d == 0) return s + N * t1 + N * N * t2;
-  if (d == 1) return t1 + N * s + N * N * t2;
-  return t1 + N * t2 + N * N * s;
-}
 
 // neighbour face-point index of own face point t under the orientation bits (swap, flip1, flip2)
 template <int N>

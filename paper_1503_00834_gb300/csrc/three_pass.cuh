@@ -34,14 +34,11 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 // ------------------------------------------------------------------ division
 
 // Quotients of the point physics.  FP64: the correctly rounded quotient.  FP32 (the perturbation
-// form, whose tolerance is relative 1e-5): with kFastDivF32 the approximate quotient __fdividef
-// (reciprocal and product, error of a few ulp for divisors of normal magnitude) instead of the
-// correctly rounded division sequence.
-constexpr bool kFastDivF32 = true;
-
+// form, whose tolerance is relative 1e-5): the approximate quotient __fdividef (reciprocal and product,
+// error of a few ulp for divisors of normal magnitude).
 template <class R>
 __device__ __forceinline__ R qdiv(R a, R b) {
-  if constexpr (sizeof(R) == 4 && kFastDivF32) return __fdividef(a, b);
+  if constexpr (sizeof(R) == 4) return __fdividef(a, b);
   else return a / b;
 }
 
