@@ -280,9 +280,11 @@ chorus_status chorus_closure_attach(chorus_mesh coarse, const void* weights);
  * chorus_rk_step launch is bracketed by a pair of CUDA events recorded on the call's stream (the
  * kernels themselves are unchanged).  chorus_timing_read synchronises the stream and returns, per
  * kernel class (0: face traces, 1: the volume kernel - lifted gradients, one-sided viscous face fluxes,
- * interior fluxes, sources and RK combination, 2: the end-point fluxes added and the new state's
- * traces, 3: common fluxes of the faces), the summed device
- * milliseconds and launch counts recorded since the last read, then clears them.  ms, counts: host
+ * interior fluxes and sources, 2: the end-point fluxes added, the RK combination and the new state's
+ * traces, 3: common fluxes of the faces), the summed device milliseconds and launch counts recorded since
+ * the last read, then clears them.  In the FP32 SSP-RK(5,4) stages (scheme 1) class 1 is the lifting kernel
+ * (gradients, one-sided viscous face fluxes) and class 2 the residual kernel (all fluxes but the faces',
+ * sources, RK combination and traces).  ms, counts: host
  * arrays of 4.  enable = 0 stops recording. */
 chorus_status chorus_timing_enable(chorus_mesh mesh, int enable);
 chorus_status chorus_timing_read(chorus_mesh mesh, void* stream, double* ms, int64_t* counts);

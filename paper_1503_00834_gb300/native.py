@@ -254,8 +254,9 @@ class Mesh:
         _ok("chorus_timing_enable", load().chorus_timing_enable(self.handle, 1 if enable else 0))
 
     def timing_read(self, stream=None):
-        """(ms[4], counts[4]) per kernel class: 0 traces, 1 volume kernel, 2 update (end-point fluxes and
-        traces), 3 common face fluxes."""
+        """(ms[4], counts[4]) per kernel class: 0 traces, 1 volume kernel, 2 update (end-point fluxes, RK
+        combination and traces), 3 common face fluxes; in FP32 SSP-RK(5,4) stages 1 lifting kernel, 2
+        residual kernel."""
         ms = (ctypes.c_double * 4)()
         cnt = (ctypes.c_int64 * 4)()
         _ok("chorus_timing_read", load().chorus_timing_read(self.handle, _stream(stream), ms, cnt))
