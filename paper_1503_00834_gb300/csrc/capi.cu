@@ -466,13 +466,20 @@ void free_mesh(chorus_mesh_s* m) {
   delete m;
 }
 
-size_t ws_words(const chorus_mesh_s* m) {
+// Words an element of the workspace's block G: the gradient record of the FP32 three-pass kernels
+// (12 N^3), or what the other stages keep there, the partial residual and the marks of the elements to skip.
+size_t record_words(const chorus_mesh_s* m, size_t word) {
+  const size_t N3 = (size_t)m->N * m->N * m->N;
+  return word == sizeof(double) ? 5 * N3 + 1 : 12 * N3;
+}
+
+// Bytes of the workspace for values of `word` bytes.
+size_t ws_bytes(const chorus_mesh_s* m, size_t word) {
   const size_t N = m->N, E = m->E;
   const size_t N2 = N * N, N3 = N2 * N;
   // stage buffer + two trace buffers + one-sided viscous face fluxes + two more stage buffers (RK(5,4))
-  // + the gradient record of the three-pass kernels, where the other stages keep the partial residual and
-  // the marks of the elements to skip + the common face fluxes of every face point
-  return 3 * E * 5 * N3 + 2 * E * 6 * 5 * N2 + E * 6 * 4 * N2 + E * 12 * N3 + E * 6 * 5 * N2;
+  // + block G + the common face fluxes of every face point
+  return (3 * E * 5 * N3 + 2 * E * 6 * 5 * N2 + E * 6 * 4 * N2 + E * record_words(m, word) + E * 6 * 5 * N2) * word + 256;
 }
 
 template <class R>
@@ -502,7 +509,7 @@ Ws<R> split_ws(const chorus_mesh_s* m, void* w) {
   r.A = r.Tv + E * 6 * 4 * N2;
   r.B = r.A + E * 5 * N3;
   r.G = r.B + E * 5 * N3;
-  r.Fc = r.G + E * 12 * N3;
+  r.Fc = r.G + E * record_words(m, sizeof(R));
   r.part = r.G;
   r.skip = (int*)(r.part + E * 5 * N3);
   return r;
@@ -718,7 +725,7 @@ chorus_status chorus_mesh_info(chorus_mesh m, int64_t* n_dof, int64_t* n_faces, 
 
 size_t chorus_rk_workspace_bytes(chorus_mesh m, chorus_precision prec) {
   if (!m) return 0;
-  return ws_words(m) * (prec == CHORUS_FP64 ? sizeof(double) : sizeof(float)) + 256;
+  return ws_bytes(m, prec == CHORUS_FP64 ? sizeof(double) : sizeof(float));
 }
 
 }  // extern "C"
