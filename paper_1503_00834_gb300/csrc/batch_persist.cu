@@ -77,6 +77,8 @@ __device__ __noinline__ void trace_item(const PersistArgs& P, int64_t t) {
 }
 template <int S>
 __device__ __noinline__ void vol_item(const PersistArgs& P, int64_t t, uint64_t* bar, uint32_t& pbar) {
+  stage_tables<S + 3, true, float, p_epb<S>(), kPThreads>(P.vol[S]);  // the tile before may have been of another order
+  __syncthreads();
   vol_tile<S + 3, true, float, p_epb<S>(), false>(P.vol[S], t, bar, pbar);
 }
 template <int S>

@@ -112,11 +112,11 @@ struct Layout {
   // banks (0.206 -> 0.193 ms at 98,304 elements); no stride measured better at N = 5 and 6
   static constexpr int SG = padded ? pad_stride<R>(16 * N3) : 16 * N3 + (N == 3 && sizeof(R) == 4 ? 11 : 0);
   // interpolation I[f][s], then derivative D[i][f] as [f][i], as pairs of equal values, indexed by rolled
-  // loops; a table for each unit (only its own threads wait for its stores)
+  // loops (stage_tables)
   static constexpr int TAB = 4 * (N + 1) * N;
   static constexpr int units = (EPB + unit_elems<N, EPB>() - 1) / unit_elems<N, EPB>();
   static constexpr int oI = 0;
-  static constexpr int oQ = (oI + units * TAB + 31) / 32 * 32;
+  static constexpr int oQ = (oI + TAB + 31) / 32 * 32;
   static constexpr int oBG = oQ + block(5 * N3);
   static constexpr int oGR0 = oBG + (PERT ? block(2 * N3) : 0);
   static constexpr int oG = oGR0 + (PERT ? block(3 * N3) : 0);
@@ -852,14 +852,27 @@ __device__ __forceinline__ void add_div(const Elem<R>& x, int ln, const R (&acc)
 // ------------------------------------------------------------------ volume kernel
 
 // Bound by instruction issue and the latency of dependent instructions at the warps that registers
-// allow: at p = 3 in FP32 (331,776 elements) 1.15 ms for 13.6 KB of DRAM traffic an element, 58 % of the
-// issue slots at 12 warps per SM, DRAM at 46 %; the lifting and residual kernels that it replaces took 1.97 ms,
-// 28.9 KB and 1.4 times the instructions.  p = 2 (98,304 elements) 0.52 -> 0.18 ms, p = 4 (111,078) 2.92 ->
-// 0.97 ms (shared-memory pipe 62 %), p = 5 (98,304) 3.34 -> 1.85 ms; FP64 at p = 3 43.7 -> 31.9 ms, at the
+// allow: at p = 3 in FP32 (331,776 elements) 1.14 ms for 12.2 KB of DRAM traffic an element, 58 % of the
+// issue slots at 12 warps per SM, DRAM at 43 %; the lifting and residual kernels that it replaces took 1.97 ms,
+// 28.9 KB and 1.5 times the instructions.  p = 2 (98,304 elements) 0.52 -> 0.18 ms, p = 4 (111,078) 2.92 ->
+// 0.97 ms (shared-memory pipe 63 %), p = 5 (98,304) 3.34 -> 1.85 ms; FP64 at p = 3 43.7 -> 31.9 ms, at the
 // FP64 units' rate.
 
 // Barriers of a unit: the staging, the two refills of the metric buffers, and the epilogue's inputs.
 constexpr int kVolBars = 4;
+
+// The operator tables of a CTA's tiles, each value as a pair; a CTA barrier follows before the tiles read
+// them.  (A table for each staging unit, stored in vol_tile, needs no barrier but measured slower: p = 3,
+// 4,800 elements 38.1 -> 39.4 us a stage, 98,304 elements 575 -> 578.)  NT: threads of the CTA.
+template <int N, bool PERT, class R, int EPB, int NT>
+__device__ __forceinline__ void stage_tables(const KArgs<R>& A) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  R* tab = reinterpret_cast<R*>(smem_raw) + Layout<N, PERT, R, EPB>::oI;
+  for (int i = threadIdx.x; i < 2 * (N + 1) * N; i += NT) {
+    const R w = __ldg(A.m.tab + i);
+    *reinterpret_cast<Pair<R>*>(tab + 2 * i) = Pair<R>{w, w};
+  }
+}
 
 // Tile `tile` (elements tile * EPB ...; threads beyond EPB * N^2 idle but take part in the barriers).
 // bars: the CTA's barriers, kVolBars for each unit (initialised), pbar: the parity of their next phase.
@@ -882,17 +895,12 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
   if (ne == 0) return;  // the same in every thread of the unit
   const uint32_t polls = wait_polls(A.err);
   const uint32_t par = pbar;
-  R* tab = sm + L::oI + unit * L::TAB;
+  const R* tab = sm + L::oI;
   LiftPre<N, R, L::SM> pre[L::SM ? 3 : 1];
   int nbr[6] = {0, 0, 0, 0, 0, 0};
   if (active) load_six(A.m.nbr, e, nbr);
   Shift sh;
   if (!stage_elements<N, PERT, R, EPB>(A, sm, bar, pbar, e0, ne, u0, tid, UT, sh, polls, [&] {
-        // operator tables, each value as a pair
-        for (int i = tid; i < 2 * (N + 1) * N; i += UT) {
-          const R w = __ldg(A.m.tab + i);
-          *reinterpret_cast<Pair<R>*>(tab + 2 * i) = Pair<R>{w, w};
-        }
         if (!active) return;
         lift_prefetch<N, R, 2, L::SM>(A, e, ln, pre[0], nbr);
         if constexpr (L::SM) {
@@ -1048,6 +1056,7 @@ __global__ void __launch_bounds__(EPB * N * N, sizeof(R) == 4 ? vol_min_blocks<N
   __shared__ __align__(8) uint64_t bars[units * kVolBars];
   pdl_trigger();
   if (threadIdx.x < units * kVolBars) mbar_init(&bars[threadIdx.x]);
+  stage_tables<N, PERT, R, EPB, EPB * N * N>(A);
   __syncthreads();
   uint32_t ph = 0;
   vol_tile<N, PERT, R, EPB, KR>(A, blockIdx.x, bars, ph);
@@ -1144,7 +1153,7 @@ struct UpLayout {
 // The end-point fluxes' part of the divergence, added to the volume kernel's partial residual; in RK mode
 // the stage's combination and the traces of the new state.  Thread ln takes the points ln + N^2 i of its
 // element.  An element for which the volume kernel gave up a wait is left as it is.  Bound by DRAM: at p = 3,
-// 331,776 elements, 7.3 KB an element in 0.410 ms, 87 % of the copy rate.  One point's inputs are loaded while the
+// 331,776 elements, 7.5 KB an element in 0.410 ms, 89 % of the copy rate.  One point's inputs are loaded while the
 // point before is worked on: all of them ahead took 96 registers, which slowed the kernel (0.590 ms) and, no
 // room being left for its early start, a stage of 1,470 elements too (20.4 -> 26.2 us).
 template <int N, class R, int EPB, int MODE>
