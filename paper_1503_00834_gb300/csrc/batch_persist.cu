@@ -87,7 +87,7 @@ __device__ __noinline__ void face_item(const PersistArgs& P, int64_t t) {
 }
 template <int S>
 __device__ __noinline__ void update_item(const PersistArgs& P, int64_t t) {
-  update_tile<S + 3, float, p_epb<S>(), kModeRK>(P.update[S], t);
+  update_tile<S + 3, float, p_epb<S>(), kModeRK, false>(P.update[S], t);
 }
 // Each order has barriers and a parity of its own: the orders use different numbers of them (a warp's
 // own at N = 4, the staging's alone at N = 5 and 6), so after an item of one order another order's
@@ -209,6 +209,7 @@ chorus_status persist_rk3_step(StagePtrs* const groups[4], double dt, unsigned* 
       f.m = G.m; f.ph = G.ph; f.bg = G.bg; f.T = Tc; f.Tv = G.Tv; f.Fc_out = G.Fc; f.err = err;
       KArgs<float>& r = P.update[s];
       r.m = G.m; r.ops = G.ops; r.Fc = G.Fc; r.part = G.part; r.q = G.buf[sg.src]; r.out = G.buf[sg.dst];
+      r.r0 = G.bg.R0;
       r.T_out = k + 1 < (int)stg.size() ? Tn : nullptr;
       r.un = G.buf[sg.un]; r.a = (float)sg.a; r.b = (float)sg.b; r.c = (float)sg.c;
       r.dt = (float)dt; r.skip = G.skip;

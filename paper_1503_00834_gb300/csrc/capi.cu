@@ -912,11 +912,11 @@ chorus_status chorus_residual(chorus_mesh m, const chorus_params* P, chorus_prec
     }
     CHK(timed(m, 0, st, [&] { return m->L.trace64(ma, m->ops64, (const double*)Q, w.Ta, st); }));
     CHK(timed(m, 1, st, [&] {
-      return m->L.vol64(ma, m->ops64, ph, (const double*)Q, w.Ta, w.Tv, (double*)R, rc.radd, w.skip, m->d_err, st);
+      return m->L.vol64(ma, m->ops64, ph, (const double*)Q, w.Ta, w.Tv, (double*)R, w.skip, m->d_err, st);
     }));
     CHK(timed(m, 3, st, [&] { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
     CHK(timed(m, 2, st, [&] {
-      return m->L.update64(ma, m->ops64, nullptr, (const double*)R, w.Fc, (double*)R, nullptr, rc, 0.0, kModeResidual,
+      return m->L.update64(ma, m->ops64, nullptr, (const double*)R, w.Fc, (double*)R, nullptr, rc, nullptr, 0.0, kModeResidual,
                            w.skip, st);
     }));
     return CHORUS_OK;
@@ -936,11 +936,11 @@ chorus_status chorus_residual(chorus_mesh m, const chorus_params* P, chorus_prec
   }
   CHK(timed(m, 0, st, [&] { return m->L.trace32(ma, m->ops32, (const float*)Q, w.Ta, st); }));
   CHK(timed(m, 1, st, [&] {
-    return m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, (float*)R, rc.radd, w.skip, m->d_err, st);
+    return m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, w.Ta, w.Tv, (float*)R, w.skip, m->d_err, st);
   }));
   CHK(timed(m, 3, st, [&] { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, w.Ta, w.Tv, w.Fc, st); }));
   CHK(timed(m, 2, st, [&] {
-    return m->L.update32(ma, m->ops32, nullptr, (const float*)R, w.Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual,
+    return m->L.update32(ma, m->ops32, nullptr, (const float*)R, w.Fc, (float*)R, nullptr, rc, bg.R0, 0.0f, kModeResidual,
                          w.skip, st);
   }));
   return CHORUS_OK;
@@ -988,7 +988,7 @@ chorus_status run_rk(chorus_mesh_s* m, R* u, const Ws<R>& w, double dt, int64_t 
                             m->closure_buf, m->E, 0, m->d_err, st));
         c.radd = (const R*)m->closure_buf;
       }
-      CHK(timed(m, 1, st, [&] { return vol(buf[g.src], Tc, c.radd); }));
+      CHK(timed(m, 1, st, [&] { return vol(buf[g.src], Tc); }));
       CHK(timed(m, 3, st, [&] { return face(Tc); }));
       // the traces of the call's last state are read by nobody: the next call starts with its own
       R* T_out = n + 1 == n_steps && &g == &stg.back() ? nullptr : Tn;
@@ -1048,13 +1048,13 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
   bool copied = false;  // the chunks of the last stage copied the state out
   const chorus_status s = run_rk<float>(
       m, Qd, w, dt, n_steps, 0, st,
-      [&](const float* q, const float* T, const float* radd) {
-        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, w.part, radd, w.skip, m->d_err, st);
+      [&](const float* q, const float* T) {
+        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, w.part, w.skip, m->d_err, st);
       },
       [&](const float* T) { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
       [&](const float* q, float* dst, float* Tn, const RkCoef<float>& c) -> cudaError_t {
         if (++stage < last || dst != Qd)
-          return m->L.update32(ma, m->ops32, q, w.part, w.Fc, dst, Tn, c, (float)dt, kModeRK, w.skip, st);
+          return m->L.update32(ma, m->ops32, q, w.part, w.Fc, dst, Tn, c, bg.R0, (float)dt, kModeRK, w.skip, st);
         for (int k = 0; k < kHostChunks; ++k) {
           int64_t e0, ne;
           range(k, &e0, &ne);
@@ -1062,10 +1062,11 @@ chorus_status rk_step_host_fp32(chorus_mesh_s* m, const chorus_params& P, float*
           RkCoef<float> ck = c;
           const int64_t o5 = e0 * 5 * N3;
           ck.un = c.un ? c.un + o5 : nullptr;
+          ck.radd = c.radd ? c.radd + o5 : nullptr;
           ck.un2 = c.un2 ? c.un2 + o5 : nullptr;
           ck.out2 = c.out2 ? c.out2 + o5 : nullptr;
           cudaError_t e = m->L.update32(mesh_range(ma, e0, ne, N), m->ops32, q + o5, w.part + o5, w.Fc, dst + o5, Tn, ck,
-                                        (float)dt, kModeRK, w.skip + e0, st);
+                                        bg.R0 ? bg.R0 + o5 : nullptr, (float)dt, kModeRK, w.skip + e0, st);
           if (e == cudaSuccess) e = cudaEventRecord(m->copy_ev[k], st);
           if (e == cudaSuccess) e = cudaStreamWaitEvent(m->copy_stream, m->copy_ev[k], 0);
           if (e == cudaSuccess)
@@ -1158,12 +1159,12 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
     Ws<double> w = split_ws<double>(m, workspace);
     return run_rk<double>(
         m, (double*)Q, w, dt, n_steps, scheme, st,
-        [&](const double* q, const double* T, const double* radd) {
-          return m->L.vol64(ma, m->ops64, ph, q, T, w.Tv, w.part, radd, w.skip, m->d_err, st);
+        [&](const double* q, const double* T) {
+          return m->L.vol64(ma, m->ops64, ph, q, T, w.Tv, w.part, w.skip, m->d_err, st);
         },
         [&](const double* T) { return m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
         [&](const double* q, double* dst, double* Tn, const RkCoef<double>& c) {
-          return m->L.update64(ma, m->ops64, q, w.part, w.Fc, dst, Tn, c, dt, kModeRK, w.skip, st);
+          return m->L.update64(ma, m->ops64, q, w.part, w.Fc, dst, Tn, c, nullptr, dt, kModeRK, w.skip, st);
         },
         [&](const double* q, double* T) { return m->L.trace64(ma, m->ops64, q, T, st); });
   }
@@ -1180,7 +1181,7 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
     bg.bgT = m->d_bgTo;
     return run_rk<float>(
         m, (float*)Q, w, dt, n_steps, scheme, st,
-        [&](const float* q, const float* T, const float*) {
+        [&](const float* q, const float* T) {
           return m->L3.grad(ma, m->ops32, ph, bg, q, T, w.Tv, w.G, m->d_err, st);
         },
         [&](const float* T) {
@@ -1193,12 +1194,12 @@ chorus_status chorus_rk_step_scheme(chorus_mesh m, const chorus_params* P, choru
   }
   return run_rk<float>(
       m, (float*)Q, w, dt, n_steps, scheme, st,
-      [&](const float* q, const float* T, const float* radd) {
-        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, w.part, radd, w.skip, m->d_err, st);
+      [&](const float* q, const float* T) {
+        return m->L.vol32(ma, m->ops32, ph, bg, q, T, w.Tv, w.part, w.skip, m->d_err, st);
       },
       [&](const float* T) { return m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, w.Tv, w.Fc, st); },
       [&](const float* q, float* dst, float* Tn, const RkCoef<float>& c) {
-        return m->L.update32(ma, m->ops32, q, w.part, w.Fc, dst, Tn, c, (float)dt, kModeRK, w.skip, st);
+        return m->L.update32(ma, m->ops32, q, w.part, w.Fc, dst, Tn, c, bg.R0, (float)dt, kModeRK, w.skip, st);
       },
       [&](const float* q, float* T) { return m->L.trace32(ma, m->ops32, q, T, st); });
 }
@@ -1605,9 +1606,9 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
       rc.radd = (const double*)m->closure_buf;
     }
     CHK(m->L.trace64(ma, m->ops64, (const double*)Q, T, st));
-    CHK(m->L.vol64(ma, m->ops64, ph, (const double*)Q, T, Tv, (double*)R, rc.radd, skip, m->d_err, st));
+    CHK(m->L.vol64(ma, m->ops64, ph, (const double*)Q, T, Tv, (double*)R, skip, m->d_err, st));
     CHK(m->L.face64(ma, ph, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st));
-    CHK(m->L.update64(ma, m->ops64, nullptr, (const double*)R, Fc, (double*)R, nullptr, rc, 0.0, kModeResidual, skip,
+    CHK(m->L.update64(ma, m->ops64, nullptr, (const double*)R, Fc, (double*)R, nullptr, rc, nullptr, 0.0, kModeResidual, skip,
                       st));
     return CHORUS_OK;
   }
@@ -1624,9 +1625,9 @@ extern "C" chorus_status chorus_residual_noalloc(chorus_mesh m, const chorus_par
     rc.radd = (const float*)m->closure_buf;
   }
   CHK(m->L.trace32(ma, m->ops32, (const float*)Q, T, st));
-  CHK(m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, (float*)R, rc.radd, skip, m->d_err, st));
+  CHK(m->L.vol32(ma, m->ops32, ph, bg, (const float*)Q, T, Tv, (float*)R, skip, m->d_err, st));
   CHK(m->L.face32(ma, ph, bg, m->d_faces, m->n_ifaces, m->n_wfaces, T, Tv, Fc, st));
-  CHK(m->L.update32(ma, m->ops32, nullptr, (const float*)R, Fc, (float*)R, nullptr, rc, 0.0f, kModeResidual, skip, st));
+  CHK(m->L.update32(ma, m->ops32, nullptr, (const float*)R, Fc, (float*)R, nullptr, rc, bg.R0, 0.0f, kModeResidual, skip, st));
   return CHORUS_OK;
 }
 

@@ -86,10 +86,11 @@ struct RkCoef {
 // Per-order launchers (defined in kern_p<N>.cu).  All return cudaGetLastError().
 //   trace   face traces of q, each in the neighbour's slot (trace_slot); T: of the whole mesh
 //   vol     from q and its traces: one-sided viscous face fluxes Tv and `part`, the residual without the
-//           end-point fluxes; radd: an additive residual correction (e.g. the learned closure) or null
+//           end-point fluxes
 //   face    common fluxes Fc [faces][5][N^2], along the owner's outward S, of the face list (n_faces
 //           interior faces, from their lower element, then n_walls wall faces)
-//   update  `out` from `part` and the end-point fluxes: the residual (mode kModeResidual; `out` may be
+//   update  `out` from `part`, the end-point fluxes, r0 (R(Q0) or null; added by vol or update, by the order)
+//           and rk.radd: the residual (mode kModeResidual; `out` may be
 //           `part`) or the stage state (kModeRK, and rk.out2; `out` may be q or rk.un), with T_out its
 //           traces (of the whole mesh)
 // skip [E]: vol marks the elements whose staging gave up (it stores nothing for them), update leaves
@@ -97,22 +98,21 @@ struct RkCoef {
 struct LaunchSet {
   cudaError_t (*trace64)(const MeshArg<double>&, const OpsArg<double>&, const double* q, double* T, cudaStream_t);
   cudaError_t (*vol64)(const MeshArg<double>&, const OpsArg<double>&, const PhysArg<double>&, const double* q,
-                       const double* T, double* Tv, double* part, const double* radd, int* skip, unsigned* err,
-                       cudaStream_t);
+                       const double* T, double* Tv, double* part, int* skip, unsigned* err, cudaStream_t);
   cudaError_t (*face64)(const MeshArg<double>&, const PhysArg<double>&, const int2* faces, int n_faces, int n_walls,
                         const double* T, const double* Tv, double* Fc, cudaStream_t);
   cudaError_t (*update64)(const MeshArg<double>&, const OpsArg<double>&, const double* q, const double* part,
-                          const double* Fc, double* out, double* T_out, const RkCoef<double>& rk, double dt, int mode,
-                          const int* skip, cudaStream_t);
+                          const double* Fc, double* out, double* T_out, const RkCoef<double>& rk, const double* r0,
+                          double dt, int mode, const int* skip, cudaStream_t);
   cudaError_t (*trace32)(const MeshArg<float>&, const OpsArg<float>&, const float* q, float* T, cudaStream_t);
   cudaError_t (*vol32)(const MeshArg<float>&, const OpsArg<float>&, const PhysArg<float>&, const BgArg&,
-                       const float* q, const float* T, float* Tv, float* part, const float* radd, int* skip,
-                       unsigned* err, cudaStream_t);
+                       const float* q, const float* T, float* Tv, float* part, int* skip, unsigned* err,
+                       cudaStream_t);
   cudaError_t (*face32)(const MeshArg<float>&, const PhysArg<float>&, const BgArg&, const int2* faces, int n_faces,
                         int n_walls, const float* T, const float* Tv, float* Fc, cudaStream_t);
   cudaError_t (*update32)(const MeshArg<float>&, const OpsArg<float>&, const float* q, const float* part,
-                          const float* Fc, float* out, float* T_out, const RkCoef<float>& rk, float dt, int mode,
-                          const int* skip, cudaStream_t);
+                          const float* Fc, float* out, float* T_out, const RkCoef<float>& rk, const float* r0,
+                          float dt, int mode, const int* skip, cudaStream_t);
   int epb32;  // elements per CTA of the FP32 volume kernel
 };
 

@@ -14,18 +14,18 @@ struct Inst {
     return Launch<N, PERT, R, EPB>::trace(m, ops, q, T, st);
   }
   static cudaError_t vol64(const MeshArg<double>& m, const OpsArg<double>& ops, const PhysArg<double>& ph,
-                           const double* q, const double* T, double* Tv, double* part, const double* radd, int* skip,
-                           unsigned* err, cudaStream_t st) {
+                           const double* q, const double* T, double* Tv, double* part, int* skip, unsigned* err,
+                           cudaStream_t st) {
     KArgs<double> A{};
-    A.m = m; A.ops = ops; A.ph = ph; A.q = q; A.T = T; A.Tv_out = Tv; A.part_out = part; A.radd = radd;
+    A.m = m; A.ops = ops; A.ph = ph; A.q = q; A.T = T; A.Tv_out = Tv; A.part_out = part;
     A.skip_out = skip; A.err = err;
     return Launch<N, false, double, EPB64>::vol(A, st);
   }
   static cudaError_t vol32(const MeshArg<float>& m, const OpsArg<float>& ops, const PhysArg<float>& ph,
-                           const BgArg& bg, const float* q, const float* T, float* Tv, float* part, const float* radd,
-                           int* skip, unsigned* err, cudaStream_t st) {
+                           const BgArg& bg, const float* q, const float* T, float* Tv, float* part, int* skip,
+                           unsigned* err, cudaStream_t st) {
     KArgs<float> A{};
-    A.m = m; A.ops = ops; A.ph = ph; A.bg = bg; A.q = q; A.T = T; A.Tv_out = Tv; A.part_out = part; A.radd = radd;
+    A.m = m; A.ops = ops; A.ph = ph; A.bg = bg; A.q = q; A.T = T; A.Tv_out = Tv; A.part_out = part;
     A.skip_out = skip; A.err = err;
     return Launch<N, true, float, EPB32>::vol(A, st);
   }
@@ -43,13 +43,14 @@ struct Inst {
   }
   template <bool PERT, class R, int EPB>
   static cudaError_t update(const MeshArg<R>& m, const OpsArg<R>& ops, const R* q, const R* part, const R* Fc, R* out,
-                            R* T_out, const RkCoef<R>& rk, R dt, int mode, const int* skip, cudaStream_t st) {
+                            R* T_out, const RkCoef<R>& rk, const R* r0, R dt, int mode, const int* skip,
+                            cudaStream_t st) {
     using L = Launch<N, PERT, R, EPB>;
     KArgs<R> A{};
     A.m = m; A.ops = ops; A.q = q; A.part = part; A.Fc = Fc; A.out = out; A.T_out = T_out;
     A.un = rk.un; A.a = rk.a; A.b = rk.b; A.c = rk.c;
     A.un2 = rk.un2; A.out2 = rk.out2; A.a2 = rk.a2; A.b2 = rk.b2; A.c2 = rk.c2;
-    A.dt = dt; A.skip = skip;
+    A.radd = rk.radd; A.r0 = r0; A.dt = dt; A.skip = skip;
     return mode == kModeRK ? L::template update<kModeRK>(A, st) : L::template update<kModeResidual>(A, st);
   }
   static LaunchSet set() {

@@ -4,14 +4,15 @@
 //   k_vol     everything an element can do alone once its neighbours' traces are known: the lifted
 //             gradients, the one-sided viscous flux of every face point (written for both sides), the
 //             fluxes at the interior flux points, their part of the divergence and the sources.
-//             Writes the residual without the two end-point fluxes of each line.
+//             Writes the residual without the two end-point fluxes of each line (at p = 2 without R(Q0)
+//             either: late_background).
 //   k_face    the common flux of every face point, once per face, from both sides' traces.
 //   k_update  adds the end-point fluxes' part of the divergence, forms the RK combination and writes the
 //             new state's traces.
 // The gradient record never leaves the SM, and the metrics and the background are read once a stage.
 // The state is read again by k_update, so that the new state is rounded once, from the whole residual:
 // with the combination in k_vol and the end-point fluxes added to its rounded result (one read of the state
-// less; p = 3, 331,776 elements: 1.82 against 1.88 ms a stage) a step was 7 to 17 % further from the 64-bit
+// less; p = 3, 331,776 elements: 1.82 against 1.87 ms a stage) a step was 7 to 17 % further from the 64-bit
 // one, at every order.
 //
 // k_vol: one CTA processes EPB elements; each element is handled by N*N threads, thread `ln` owning
@@ -29,7 +30,7 @@
 // element blocks are padded so that the two elements of a warp use opposite halves of the banks, and
 // the computed arrays are XOR-swizzled so that xi-, eta- and zeta-line accesses are conflict free.
 #pragma once
-#include <type_traits>
+#include <utility>
 #include <utility>
 
 #include "sd_device.cuh"
@@ -97,6 +98,14 @@ __host__ __device__ constexpr bool stage_metrics() { return sizeof(R) == 4 && N 
 template <int N, class R>
 __host__ __device__ constexpr bool stage_epilogue() { return warp_local<N>() && reg_lines<N, R>() && stage_metrics<N, R>(); }
 
+// Whether k_update adds R(Q0) (FP32), to the whole perturbation residual, rather than k_vol to the part
+// without the end points.  A coarse p = 2 shell's residual is mostly R(Q0), and the part would be rounded at
+// that size once more (288 and 450 elements: 6 to 7 % further from the 64-bit residual than the three-pass
+// kernels'; late, as far as theirs; 98,304 elements take 334 us a stage either way).  From p = 3 on the early
+// sum is the closer one, by 2 to 3 %.
+template <int N, class R>
+__host__ __device__ constexpr bool late_background() { return sizeof(R) == 4 && N == 3; }
+
 template <int N, bool PERT, class R, int EPB>
 struct Layout {
   static constexpr int N2 = N * N, N3 = N * N * N;
@@ -151,7 +160,8 @@ struct KArgs {
   const R* un2;        // optional second output: out2 = a2 un2 + b2 q + c2 dt R
   R* out2;
   R a2, b2, c2;
-  const R* radd;       // k_vol: optional additive residual correction [E][5][N3]
+  const R* r0;         // k_update: R(Q0) [E][5][N3] where it adds it (late_background), or null
+  const R* radd;       // k_update: optional additive residual correction [E][5][N3]
   R* Fc_out;           // k_face output: common fluxes along the owner's outward S [faces][5][N2]
   const R* Fc;         // k_update input
   int* skip_out;       // k_vol: per element, 1 if its staging gave up (nothing stored for it), else 0
@@ -960,7 +970,7 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
   unit_sync<N>();
   // the epilogue's inputs: staged (SE) into the record's space (R(Q0)) and the free metric buffer (x)
   constexpr bool SE = PERT && stage_epilogue<N, R>();
-  const bool want_r0 = PERT && A.bg.R0 != nullptr;
+  const bool want_r0 = PERT && !late_background<N, R>() && A.bg.R0 != nullptr;
   const unsigned lanes = SE ? __ballot_sync(0xffffffffu, active) : 0u;
   if constexpr (PERT && !SE) {
     if (tid == 0) {
@@ -1013,41 +1023,36 @@ __device__ __forceinline__ void vol_tile(const KArgs<R>& A, int64_t tile, uint64
   };
   // residual dQ/dt = -div/|J| - M (Eqs. 4, 11) without the end points, sources of Eqs. 2-3
   const PhysArg<R>& ph = A.ph;
-  auto finish = [&](auto extra) {  // extra: an additive correction
-    In cur, nxt = load_in(0);
+  In cur, nxt = load_in(0);
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-      cur = nxt;
-      if (i + 1 < N) nxt = load_in(i + 1);
-      const int pt = ln + N2 * i;
-      const int si = sidx<N, R>(ln % N, ln / N, i);
-      R q[5];
+  for (int i = 0; i < N; ++i) {
+    cur = nxt;
+    if (i + 1 < N) nxt = load_in(i + 1);
+    const int pt = ln + N2 * i;
+    const int si = sidx<N, R>(ln % N, ln / N, i);
+    R q[5];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) q[v] = x.q[v * N3 + pt];
-      R gr = ph.GM;  // g3 points outward (the source uses -rho g_vec); FP32: x holds x / |x|^3
-      if constexpr (sizeof(R) == 8) {
-        const R r2 = dot3(cur.x, cur.x);
-        gr *= qrcp(r2 * sqrt(r2));
-      }
-      const R g3[3] = {gr * cur.x[0], gr * cur.x[1], gr * cur.x[2]};
-      R M[5];
-      M[0] = R(0);
-      M[1] = q[0] * g3[0] - ph.twoOmega * q[2];
-      M[2] = q[0] * g3[1] + ph.twoOmega * q[1];
-      M[3] = q[0] * g3[2];
-      M[4] = q[1] * g3[0] + q[2] * g3[1] + q[3] * g3[2];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        R Rv = -(x.g[(kG + v) * N3 + si] + acc[v][i]) * cur.ij - M[v];
-        if (PERT) Rv += cur.r0[v];
-        const size_t oi = ((size_t)e * 5 + v) * N3 + pt;
-        if (decltype(extra)::value) Rv += ld_written(A.radd + oi);
-        A.part_out[oi] = Rv;
-      }
+    for (int v = 0; v < 5; ++v) q[v] = x.q[v * N3 + pt];
+    R gr = ph.GM;  // g3 points outward (the source uses -rho g_vec); FP32: x holds x / |x|^3
+    if constexpr (sizeof(R) == 8) {
+      const R r2 = dot3(cur.x, cur.x);
+      gr *= qrcp(r2 * sqrt(r2));
     }
-  };
-  if (A.radd != nullptr) finish(std::true_type{});
-  else finish(std::false_type{});
+    const R g3[3] = {gr * cur.x[0], gr * cur.x[1], gr * cur.x[2]};
+    R M[5];
+    M[0] = R(0);
+    M[1] = q[0] * g3[0] - ph.twoOmega * q[2];
+    M[2] = q[0] * g3[1] + ph.twoOmega * q[1];
+    M[3] = q[0] * g3[2];
+    M[4] = q[1] * g3[0] + q[2] * g3[1] + q[3] * g3[2];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      R Rv = -(x.g[(kG + v) * N3 + si] + acc[v][i]) * cur.ij - M[v];
+      if (PERT && !late_background<N, R>()) Rv += cur.r0[v];
+      const size_t oi = ((size_t)e * 5 + v) * N3 + pt;
+      A.part_out[oi] = Rv;
+    }
+  }
 }
 
 template <int N, bool PERT, class R, int EPB, bool KR>
@@ -1151,12 +1156,12 @@ struct UpLayout {
 };
 
 // The end-point fluxes' part of the divergence, added to the volume kernel's partial residual; in RK mode
-// the stage's combination and the traces of the new state.  Thread ln takes the points ln + N^2 i of its
+// the stage's combination and the traces of the new state.  ADD: with an additive correction.  Thread ln takes the points ln + N^2 i of its
 // element.  An element for which the volume kernel gave up a wait is left as it is.  Bound by DRAM: at p = 3,
 // 331,776 elements, 7.5 KB an element in 0.410 ms, 89 % of the copy rate.  One point's inputs are loaded while the
 // point before is worked on: all of them ahead took 96 registers, which slowed the kernel (0.590 ms) and, no
 // room being left for its early start, a stage of 1,470 elements too (20.4 -> 26.2 us).
-template <int N, class R, int EPB, int MODE>
+template <int N, class R, int EPB, int MODE, bool ADD>
 __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
   using L = UpLayout<N, R, EPB>;
   constexpr int N2 = N * N, N3 = N * N * N;
@@ -1175,11 +1180,12 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
     load_six(A.m.code, e, code);
     load_six(A.m.fid, e, fid);
   }
+  constexpr bool LATE = late_background<N, R>();
   pdl_wait();
   const int skip = active ? ld_written(A.skip + e) : 1;
   // A point's inputs, loaded one point ahead.
   struct In {
-    R ij, part[5], q[NI], un[NI];
+    R ij, part[5], q[NI], un[NI], add[ADD ? 5 : 1], r0[LATE ? 5 : 1];
   };
   auto load_in = [&](int i) {
     In in;
@@ -1188,6 +1194,8 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
     for (int v = 0; v < 5; ++v) {
       const size_t oi = ((size_t)e * 5 + v) * N3 + ln + N2 * i;
       in.part[v] = ld_written(A.part + oi);
+      if constexpr (ADD) in.add[v] = ld_written(A.radd + oi);
+      if constexpr (LATE) in.r0[v] = A.r0 != nullptr ? __ldg(A.r0 + oi) : R(0);
       if constexpr (MODE == kModeRK) {
         in.q[v] = ld_written(A.q + oi);
         in.un[v] = A.a != R(0) ? ld_written(A.un + oi) : R(0);  // a stage without a u^n term does not read it
@@ -1232,7 +1240,9 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
         s += d0b * sF[(10 + v) * N2 + a + N * i] + dNb * sF[(15 + v) * N2 + a + N * i];
         s *= in.ij;
         const size_t oi = ((size_t)e * 5 + v) * N3 + pt;
-        R w = in.part[v] - s;  // the whole residual
+        R w = in.part[v] - s;
+        if constexpr (LATE) w += in.r0[v];
+        if constexpr (ADD) w += in.add[v];  // the whole residual
         if constexpr (MODE == kModeRK) {
           const R dR = A.dt * w, bq = A.b * in.q[v];
           if (A.out2) A.out2[oi] = fma_rn(A.c2, dR, fma_rn(A.a2, A.un2[oi], A.b2 * in.q[v]));
@@ -1272,10 +1282,10 @@ __device__ __forceinline__ void update_tile(const KArgs<R>& A, int64_t tile) {
   }
 }
 
-template <int N, class R, int EPB, int MODE>
+template <int N, class R, int EPB, int MODE, bool ADD>
 __global__ void __launch_bounds__(EPB * N * N) k_update(const KArgs<R> A) {
   pdl_trigger();
-  update_tile<N, R, EPB, MODE>(A, blockIdx.x);
+  update_tile<N, R, EPB, MODE, ADD>(A, blockIdx.x);
 }
 
 // ------------------------------------------------------------------ launch helpers
@@ -1345,10 +1355,20 @@ struct Launch {
     if (A.m.E == 0) return cudaSuccess;
     if (A.Fc == nullptr || A.part == nullptr || A.out == nullptr || A.skip == nullptr) return cudaErrorInvalidValue;
     if (MODE == kModeRK && (A.q == nullptr || (A.a != R(0) && A.un == nullptr))) return cudaErrorInvalidValue;
+    // the learned closure's order; a kernel of its own, since a test of radd at each point kept the loads of the
+    // next from starting early (331,776 elements at p = 3: 1.87 -> 1.99 ms a stage)
+    if constexpr (N == 3) {
+      if (A.radd != nullptr) return update_add<MODE, true>(A, st);
+    }
+    return A.radd != nullptr ? cudaErrorInvalidValue : update_add<MODE, false>(A, st);
+  }
+  template <int MODE, bool ADD>
+  static cudaError_t update_add(const KArgs<R>& A, cudaStream_t st) {
     const size_t sm = (size_t)UpLayout<N, R, EPB>::total * sizeof(R);
-    cudaError_t e = cudaFuncSetAttribute(k_update<N, R, EPB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    auto* k = k_update<N, R, EPB, MODE, ADD>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    return launch_dependent(early(A.m.E), k_update<N, R, EPB, MODE>, blocks(A.m.E), threads, sm, st, A);
+    return launch_dependent(early(A.m.E), k, blocks(A.m.E), threads, sm, st, A);
   }
 };
 
